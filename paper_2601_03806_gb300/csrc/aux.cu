@@ -4,11 +4,13 @@
 // reductions.
 #include <cuda_fp16.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "internal.h"
 #include "stats.cuh"
 #include "lattice.cuh"
+#include "step_kernel.cuh"
 
 namespace flbm {
 
@@ -320,6 +322,138 @@ __global__ void k_shells(const T *spec, BoxDesc b, int nshell, double *S, unsign
     }
 }
 
+// Training pairs: for every node the features x_i = g_i / sqrt(rho0 kT w_i /
+// c_s^2), x_27 = omega - 1, and the targets
+//   t_i = w_i sum_{k >= 10} e_ki rho u^(deg k) / b_k / (w_i sigma^3),
+// the ghost equilibrium content by which the regularized collision (Reg-FLBM)
+// differs from the GMF collision of the same pre-collision state, in FP64.
+//
+// The FP64 pipe bounds it (two operations per clock and SM), so the kernel is
+// arranged around its count, about 270 a node instead of 1044: the density
+// and momentum come from axis-wise partial sums (49 additions, not 81); the
+// 17 ghost amplitudes are products of per-axis factors kappa_a u^a; the
+// synthesis skips the modes below order 3; 1 / w_i, a power of four times a
+// constant, goes into the amplitudes and, exactly, into the FP32 results;
+// and 1 / sqrt(w_i) into four host constants.  A CTA's rows of X and T are
+// contiguous, so they leave through shared memory in whole lines.
+struct PairConst {
+    double x[4];        // 1 / sqrt(rho0 kT w / c_s^2) for |c|^2 = 0, 1, 2, 3
+    double scale;       // 27/8 / sigma^3: 1 / w_i = 27/8 4^(|c|^2)
+    float x27;          // omega - 1
+};
+
+// 1-D synthesis (step_kernel.cuh) of a line whose degree-0 (and, with Z1,
+// degree-1) amplitude is zero.
+template <bool Z1>
+__device__ __forceinline__ void synthesise_high(double &p0, double &p1, double &p2)
+{
+    const double t = p2, z = -2.0 * p2;
+    p0 = Z1 ? t : t - p1;
+    p2 = Z1 ? t : t + p1;
+    p1 = z;
+}
+
+constexpr int kPairBlock = 128;
+
+template <typename S>
+__global__ void __launch_bounds__(kPairBlock) k_mlp_pairs(const S *__restrict__ g, const BoxDesc b, const PairConst c,
+                                                          float *__restrict__ X, float *__restrict__ T)
+{
+    __shared__ float row[kPairBlock * 28];
+    for (uint64_t n0 = uint64_t(blockIdx.x) * kPairBlock; n0 < b.n; n0 += uint64_t(gridDim.x) * kPairBlock) {
+        const uint64_t n = n0 + threadIdx.x;
+        const uint32_t live = uint32_t(b.n - n0 < kPairBlock ? b.n - n0 : kPairBlock);
+        const bool on = threadIdx.x < live;
+        double d[3][3][3];
+        uint32_t x, y, z;
+        node_xyz(on ? n : n0, b, x, y, z);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    d[i][j][k] = ldd(g, storage_index(i - 1, j - 1, k - 1, x, y, z, b));
+                    row[threadIdx.x * 28 + slot_of(i - 1, j - 1, k - 1)] =
+                        float(d[i][j][k] * c.x[(i != 1) + (j != 1) + (k != 1)]);
+                }
+        row[threadIdx.x * 28 + 27] = c.x27;
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < live * 28; e += kPairBlock) X[n0 * 28 + e] = row[e];
+        // rho and j from sums along x, then y, then z
+        double sx[3][3], dx[3], s[3], jx = 0.0, jy = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            double m[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                sx[j][k] = (d[0][j][k] + d[2][j][k]) + d[1][j][k];
+                m[j] = d[2][j][k] - d[0][j][k];
+            }
+            dx[k] = (m[0] + m[2]) + m[1];
+            s[k] = (sx[0][k] + sx[2][k]) + sx[1][k];
+            jy += sx[2][k] - sx[0][k];
+        }
+        jx = (dx[0] + dx[2]) + dx[1];
+        const double rho = b.rho0 + ((s[0] + s[2]) + s[1]);
+        const double jz = s[2] - s[0];
+        const double ir = 1.0 / rho;
+        // per-axis factors kappa_a u^a (kappa = 2/3, 1/2, 1/2), rho and the
+        // scale in the x axis's
+        const double u[3] = {jx * ir, jy * ir, jz * ir}, r = rho * c.scale;
+        double f[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double pre = a == 0 ? r : 1.0;
+            f[a][0] = kappa1d(0) * pre;
+            f[a][1] = (kappa1d(1) * pre) * u[a];
+            f[a][2] = f[a][1] * u[a];
+        }
+        double q[3][3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const double fij = f[0][i] * f[1][j];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) q[i][j][k] = mode_order(i, j, k) >= 3 ? fij * f[2][k] : 0.0;
+            }
+        // z, y and x passes; lines and entries below order 3 are zero
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if (i + j == 1) synthesise_high<true>(q[i][j][0], q[i][j][1], q[i][j][2]);
+                else if (i + j == 2) synthesise_high<false>(q[i][j][0], q[i][j][1], q[i][j][2]);
+                else if (i + j > 2) synthesise(q[i][j][0], q[i][j][1], q[i][j][2]);
+            }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            synthesise_high<false>(q[0][0][k], q[0][1][k], q[0][2][k]);
+            synthesise(q[1][0][k], q[1][1][k], q[1][2][k]);
+            synthesise(q[2][0][k], q[2][1][k], q[2][2][k]);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) synthesise(q[0][j][k], q[1][j][k], q[2][j][k]);
+        __syncthreads();   // X has left the staging rows
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int far = (i != 1) + (j != 1) + (k != 1);
+                    row[threadIdx.x * 27 + slot_of(i - 1, j - 1, k - 1)] =
+                        float(q[i][j][k]) * (far == 0 ? 1.0f : far == 1 ? 4.0f : far == 2 ? 16.0f : 64.0f);
+                }
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < live * 27; e += kPairBlock) T[n0 * 27 + e] = row[e];
+        __syncthreads();   // T has left before the next nodes' X
+    }
+}
+
 __global__ void k_stats_finalize(const double *partials, int nblocks, DevStats *st, long long step,
                                  double n)
 {
@@ -405,6 +539,22 @@ cudaError_t launch_scatter_f(void *g, int prec, const BoxDesc &b, uint64_t n0, u
     with_storage(prec, [&](auto tag) {
         using S = decltype(tag);
         k_scatter_f<S><<<grid, 128, 0, s>>>(static_cast<S *>(g), b, n0, cn, in);
+    });
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_pairs(const void *g, int prec, const BoxDesc &b, double kT, double omega, float *X, float *T,
+                             cudaStream_t s)
+{
+    const int grid = grid_for(b.n, kPairBlock);
+    const double w[4] = {8.0 / 27.0, 2.0 / 27.0, 1.0 / 54.0, 1.0 / 216.0}, sig = std::sqrt(kT / b.rho0);
+    PairConst c;
+    for (int k = 0; k < 4; ++k) c.x[k] = 1.0 / std::sqrt(b.rho0 * kT * w[k] * 3.0);
+    c.scale = 3.375 / (sig * sig * sig);
+    c.x27 = float(omega - 1.0);
+    with_storage(prec, [&](auto tag) {
+        using S = decltype(tag);
+        k_mlp_pairs<S><<<grid, kPairBlock, 0, s>>>(static_cast<const S *>(g), b, c, X, T);
     });
     return cudaGetLastError();
 }

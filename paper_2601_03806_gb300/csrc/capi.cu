@@ -887,16 +887,7 @@ int flbm_mlp_pairs(flbm_ctx *c, float *dev_x, float *dev_t)
         return fail(c, FLBM_E_INVALID, "dev_x and dev_t must be device (or managed) memory");
     if (!(c->p.kT > 0.0)) return fail(c, FLBM_E_INVALID, "training pairs need kT > 0 (the feature scale)");
     if (int rc = materialise(c)) return rc;
-    int rc = ensure_pipe(c);
-    if (rc) return rc;
-    const BoxDesc b = box_of(c);
-    const int prec = prec_code(c);
-    for (uint64_t n0 = 0; n0 < c->n; n0 += c->pipe_nodes) {
-        const uint64_t cn = std::min<uint64_t>(c->pipe_nodes, c->n - n0);
-        CK(c, launch_gather_f(c->g, prec, b, n0, cn, c->pipe[0], true, c->stream));
-        CK(c, launch_mlp_pairs(c->pipe[0], cn, c->p.rho0, c->p.kT, 1.0 / c->p.tau, dev_x + n0 * 28,
-                               dev_t + n0 * 27, c->stream));
-    }
+    CK(c, launch_mlp_pairs(c->g, prec_code(c), box_of(c), c->p.kT, 1.0 / c->p.tau, dev_x, dev_t, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     return FLBM_OK;
 }

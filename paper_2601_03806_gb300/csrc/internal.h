@@ -214,11 +214,6 @@ cudaError_t launch_step_learned(float *g, const StepArgs<float> &a, const LearnA
 // Resident CTAs per SM of the learned step (1: a CTA holds all of an SM's
 // tensor memory); also sets the kernels' shared-memory attribute.
 int learned_occupancy(uint64_t n);
-// Training pairs (mlp_train.cu) of cn nodes from FP64 deviations g[27][cn]:
-// features X[cn][28] and targets T[cn][27] (device arrays).
-cudaError_t launch_mlp_pairs(const double *g, uint64_t cn, double rho0, double kT, double omega, float *X,
-                             float *T, cudaStream_t s);
-
 // Auxiliary kernels (aux.cu).  `prec` is 0 (double storage), 1 (float) or
 // 2 (half).
 struct BoxDesc {
@@ -235,6 +230,10 @@ cudaError_t launch_gather_state(const void *g, int prec, const BoxDesc &b, uint6
                                 uint64_t cn, void *out, cudaStream_t s);
 cudaError_t launch_scatter_f(void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,
                              const double *in, cudaStream_t s);
+// Training pairs of every node: features X[n][28], targets T[n][27] (device
+// arrays of floats).
+cudaError_t launch_mlp_pairs(const void *g, int prec, const BoxDesc &b, double kT, double omega, float *X, float *T,
+                             cudaStream_t s);
 cudaError_t launch_init_thermal(void *g, int prec, const BoxDesc &b, double kT, uint64_t seed,
                                 cudaStream_t s);
 cudaError_t launch_probe(const void *g, int prec, const BoxDesc &b, const long long *nodes,

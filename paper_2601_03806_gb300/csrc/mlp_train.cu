@@ -1,13 +1,5 @@
-// mlp_train.cu -- training of the learned-collision network on the GPU:
-// training pairs from a lattice state, the loss gradient (forward and
-// backward in FP32 on the CUDA cores), and Adam.
-//
-// Pairs: for every node, the features x (28) and the target
-//   t_i = w_i sum_{k >= 10} e_ki rho u^(deg k) / b_k / (w_i sigma^3),
-// the ghost equilibrium content by which the regularized collision
-// (Reg-FLBM) differs from the GMF collision of the same pre-collision state.
-// It is synthesised in FP64 with the same sum-factorised transform as the
-// step kernels (only the ghost amplitudes non-zero).
+// mlp_train.cu -- training of the learned-collision network on the GPU: the
+// loss gradient and Adam (the training pairs are made in aux.cu).
 //
 // Gradient of L = mean over samples and outputs of (y - t)^2, FP32 on the
 // CUDA cores.  A CTA takes tiles of T samples (8, 16 or 32) whose features,
@@ -714,72 +706,6 @@ __global__ void k_mlp_adam(float *__restrict__ img, float *__restrict__ m1, floa
     img[image_index(p)] -= lr_t * a / (sqrtf(b) + eps);
 }
 
-// Training pairs of cn nodes from FP64 deviations g[27][cn] (SoA, ABI order).
-__global__ void k_mlp_pairs(const double *__restrict__ g, uint64_t cn, double rho0, double inv_s_sqrt3,
-                            double inv_sig3, float x27, float *__restrict__ X, float *__restrict__ T)
-{
-    for (uint64_t k = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; k < cn;
-         k += uint64_t(gridDim.x) * blockDim.x) {
-        double rho = rho0, j[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const int i = slot_of(a - 1, b - 1, c - 1);
-                    const double d = g[uint64_t(i) * cn + k];
-                    rho += d;
-                    j[0] += d * (a - 1);
-                    j[1] += d * (b - 1);
-                    j[2] += d * (c - 1);
-                    // x_i = g_i / sqrt(rho0 kT w_i / c_s^2); w_i = w1 w1 w1
-                    X[k * 28 + i] = float(d * inv_s_sqrt3 / sqrt(w1(a - 1) * w1(b - 1) * w1(c - 1)));
-                }
-        X[k * 28 + 27] = x27;
-        const double u[3] = {j[0] / rho, j[1] / rho, j[2] / rho};
-        // ghost amplitudes Q = syn_scale * rho u^(deg), zero below order 3
-        double q[3][3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    double m = 0.0;
-                    if (mode_order(a, b, c) >= 3) {
-                        m = rho;
-                        for (int e = 0; e < a; ++e) m *= u[0];
-                        for (int e = 0; e < b; ++e) m *= u[1];
-                        for (int e = 0; e < c; ++e) m *= u[2];
-                        m *= syn_scale(a, b, c);
-                    }
-                    q[a][b][c] = m;
-                }
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) synthesise(q[a][b][0], q[a][b][1], q[a][b][2]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) synthesise(q[a][0][c], q[a][1][c], q[a][2][c]);
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) synthesise(q[0][b][c], q[1][b][c], q[2][b][c]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const int i = slot_of(a - 1, b - 1, c - 1);
-                    T[k * 27 + i] = float(q[a][b][c] * inv_sig3 / (w1(a - 1) * w1(b - 1) * w1(c - 1)));
-                }
-    }
-}
-
 // Samples per tile for batches of `count`: the smallest tile with at most
 // one per SM (a tile of 8 takes less than half the time of one of 32, so
 // spreading a small batch over more SMs wins), else 32 (twice the reuse of
@@ -937,17 +863,6 @@ cudaError_t launch_train(Scratch &sc, const Work &w, TrainArgs &a)
 }
 
 }  // namespace
-
-cudaError_t launch_mlp_pairs(const double *g, uint64_t cn, double rho0, double kT, double omega, float *X,
-                             float *T, cudaStream_t s)
-{
-    const double inv_s_sqrt3 = 1.0 / std::sqrt(rho0 * kT * 3.0);   // 1 / sqrt(rho0 kT / c_s^2)
-    const double sig = std::sqrt(kT / rho0);
-    const int grid = int(std::min<uint64_t>((cn + 127) / 128, 65535ull * 8));
-    k_mlp_pairs<<<std::max(grid, 1), 128, 0, s>>>(g, cn, rho0, inv_s_sqrt3, 1.0 / (sig * sig * sig),
-                                                  float(omega - 1.0), X, T);
-    return cudaGetLastError();
-}
 
 }  // namespace flbm
 

@@ -1,0 +1,33 @@
+"""The training pairs, where their code branches."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    from paper_2601_03806_gb300 import flbm
+    return flbm
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16", "fp64"])
+@pytest.mark.parametrize("shape,steps", [((1, 1, 1), 0), ((127, 1, 1), 1), ((43, 3, 1), 0), ((33, 5, 7), 1)])
+def test_pairs_match_oracle_at_block_edges(F, oracle_mod, prec, shape, steps):
+    """As the existing test of the pairs: FP64 results stored in FP32."""
+    import torch
+    from oracle import mlp as M
+    tau, kT, rho0 = 0.7, 1e-5, 1.1
+    box = F.Lattice(*shape, tau, kT, rho0=rho0, seed=4, scheme=F.FLBM_REG, precision=prec)
+    box.init_thermal(9)
+    box.step(steps)
+    f = box.get_populations().reshape(27, -1).T
+    n = f.shape[0]
+    x, t = torch.full((n + 1, 28), 7.0, device="cuda"), torch.full((n + 1, 27), 7.0, device="cuda")
+    box.mlp_pairs(x, t)
+    x, t = x.cpu().numpy().astype(float), t.cpu().numpy().astype(float)
+    assert (x[n] == 7).all() and (t[n] == 7).all()
+    xo = M.features(f, rho0, kT, 1.0 / tau)
+    to = np.array([M.target(v, tau, rho0, kT) for v in f])
+    assert np.abs(x[:n] - xo).max() <= 1e-6 * (1 + np.abs(xo).max())
+    assert np.abs(t[:n] - to).max() <= 2e-6 * np.abs(to).max() + 1e-7
