@@ -454,30 +454,39 @@ __global__ void __launch_bounds__(kPairBlock) k_mlp_pairs(const S *__restrict__ 
     }
 }
 
-__global__ void k_stats_finalize(const double *partials, int nblocks, DevStats *st, long long step,
-                                 double n)
+// Totals of the fused reductions of up to kStatSlots steps: CTA (s, i) adds
+// sum s of slot i's per-CTA partials in a fixed order, and the CTA that
+// finishes last (no CTA waits) adds the steps to the accumulators in step
+// order, a thread per component.  One launch per kStatSlots steps, and 13
+// CTAs per step because FP64 adds run at two per clock and SM: one CTA per
+// step took 15-17 us a step, a seventh of the 128^3 step and most of the 64^3
+// one; this takes about 5 us per launch.
+constexpr int kStatThreads = 128;
+__global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch f, DevStats *st, double n)
 {
-    __shared__ double red[NSTAT][256];
-    double loc[NSTAT];
-#pragma unroll
-    for (int s = 0; s < NSTAT; ++s) loc[s] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int s = 0; s < NSTAT; ++s) loc[s] += partials[size_t(b) * NSTAT + s];
-#pragma unroll
-    for (int s = 0; s < NSTAT; ++s) red[s][threadIdx.x] = loc[s];
+    __shared__ double red[kStatThreads];
+    __shared__ bool last;
+    const int s = blockIdx.x, i = blockIdx.y, t = threadIdx.x;
+    const double *p = f.partials + size_t(i) * f.slot_stride + s;
+    double v = 0.0;
+#pragma unroll 4
+    for (int b = t; b < f.nblocks[i]; b += kStatThreads) v += p[size_t(b) * NSTAT];
+    red[t] = v;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int s = 0; s < NSTAT; ++s) red[s][threadIdx.x] += red[s][threadIdx.x + w];
+    for (int w = kStatThreads / 2; w > 0; w >>= 1) {
+        if (t < w) red[t] += red[t + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        double tot[NSTAT];
-        for (int s = 0; s < NSTAT; ++s) tot[s] = red[s][0];
-        stats_update(st, tot, step, n);
+    if (t == 0) {
+        f.totals[i * NSTAT + s] = red[0];
+        __threadfence();
+        last = atomicAdd(f.arrived, 1u) == gridDim.x * gridDim.y - 1;
     }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    stats_update(st, f.totals, int(gridDim.y), f.step, n, t);
+    if (t == 0) *f.arrived = 0u;
 }
 
 inline int grid_for(uint64_t work, int block)
@@ -620,10 +629,9 @@ cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshe
     return cudaGetLastError();
 }
 
-cudaError_t launch_stats_finalize(const double *partials, int nblocks, DevStats *st, long long step,
-                                  double n, cudaStream_t s)
+cudaError_t launch_stats_finalize(const StatBatch &f, int slots, DevStats *st, double n, cudaStream_t s)
 {
-    k_stats_finalize<<<1, 256, 0, s>>>(partials, nblocks, st, step, n);
+    k_stats_finalize<<<dim3(NSTAT, unsigned(slots)), kStatThreads, 0, s>>>(f, st, n);
     return cudaGetLastError();
 }
 

@@ -186,7 +186,7 @@ void fill_constants_t(const flbm_params &p, StepArgs<R> &a)
 }
 
 template <typename R>
-StepArgs<R> make_args(const flbm_ctx *c, int64_t t)
+StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr)
 {
     StepArgs<R> a;
     std::memset(&a, 0, sizeof(a));
@@ -200,7 +200,7 @@ StepArgs<R> make_args(const flbm_ctx *c, int64_t t)
     a.step = uint64_t(t);
     fill_constants_t<R>(c->p, a);
     a.tx_pad = c->tx_pad;
-    a.partials = c->partials;
+    a.partials = partials;
     a.flag = &c->dflags->flag;
     a.bad_step = &c->dflags->bad_step;
     return a;
@@ -323,7 +323,8 @@ void flbm::destroy_ctx(flbm_ctx *c)
     delete c;
 }
 
-int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void *stream, flbm_ctx **out)
+int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void *stream, flbm_ctx **out,
+                     int stat_slots)
 {
     if (!out) return fail(nullptr, FLBM_E_INVALID, "out is NULL");
     *out = nullptr;
@@ -405,8 +406,9 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
         e = ms_prepare(p->scheme, c->nsm, make_args<float>(c, 0), c->ms_grid, c->ms_zseg);
         if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_CUDA); }
     }
-    const int max_grid = std::max(std::max(c->grid, c->row_grid), c->ms_grid);
-    e = cudaMalloc(&c->partials, size_t(max_grid) * NSTAT * sizeof(double));
+    c->max_grid = std::max(std::max(c->grid, c->row_grid), c->ms_grid);
+    c->stat_slots = stat_slots;
+    e = cudaMalloc(&c->partials, size_t(stat_slots) * (c->max_grid + 1) * NSTAT * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&c->dstats, sizeof(DevStats));
     if (e == cudaSuccess) e = cudaMalloc(&c->dflags, sizeof(DevFlags));
     if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_NOMEM); }
@@ -504,6 +506,21 @@ int flbm_step(flbm_ctx *c, int64_t n)
     if (c->ens) return fail(c, FLBM_E_INVALID, "an ensemble replica is stepped by flbm_ensemble_step");
     if (n < 0) return fail(c, FLBM_E_INVALID, "n must be >= 0");
     const int every = c->p.stats_every;
+    // reduced steps leave their partial sums in a slot each; totals are
+    // formed when the slots are full and after the last step
+    StatBatch f;
+    f.partials = c->partials;
+    f.slot_stride = size_t(c->max_grid) * NSTAT;
+    f.totals = c->partials + c->stat_slots * f.slot_stride;
+    f.arrived = &c->dflags->arrived;
+    int held = 0;
+    auto form_totals = [&] {
+        const cudaError_t e = held ? launch_stats_finalize(f, held, c->dstats, double(c->n), c->stream) : cudaSuccess;
+        held = 0;
+        return e == cudaSuccess
+                   ? FLBM_OK
+                   : fail(c, FLBM_E_CUDA, std::string("stats launch: ") + cudaGetErrorString(e));
+    };
     for (int64_t s = 0; s < n; ++s) {
         const int64_t t = c->step + s;
         const bool odd = ((t + c->phase) & 1) != 0;
@@ -519,16 +536,17 @@ int flbm_step(flbm_ctx *c, int64_t n)
             }
             CK(c, cudaEventRecord(c->ev[2 * c->ev_used], c->stream));
         }
+        double *const slot = c->partials + held * f.slot_stride;
         int reduced_grid = c->row_grid > 0 ? c->row_grid : c->grid;   // CTAs that wrote partials
         if (c->p.state_form == FLBM_STATE_MOMENTS) {
             if (!c->ms_live) {   // the first collision, from the populations
-                e = launch_ms_boot(static_cast<const float *>(c->g), c->ms[c->ms_cur], make_args<float>(c, t),
+                e = launch_ms_boot(static_cast<const float *>(c->g), c->ms[c->ms_cur], make_args<float>(c, t, slot),
                                    c->p.scheme, odd, stats, c->grid, c->stream);
                 reduced_grid = c->grid;
                 c->ms_live = true;
             } else {
                 e = launch_ms_step(c->ms[c->ms_cur], c->ms[c->ms_cur ^ 1], make_args<float>(c, t - 1),
-                                   make_args<float>(c, t), c->p.scheme, stats, c->ms_grid, c->ms_zseg,
+                                   make_args<float>(c, t, slot), c->p.scheme, stats, c->ms_grid, c->ms_zseg,
                                    c->stream);
                 reduced_grid = c->ms_grid;
                 c->ms_cur ^= 1;
@@ -543,27 +561,33 @@ int flbm_step(flbm_ctx *c, int64_t n)
             L.sig3 = float(std::pow(c->p.kT / c->p.rho0, 1.5));
             L.x27 = float(1.0 / c->p.tau - 1.0);
             L.starve = c->tx_pad != 0;   // FLBM_INJECT_STARVE=1 (tests)
-            e = launch_step_learned(static_cast<float *>(c->g), make_args<float>(c, t), L, odd, stats, c->grid,
+            e = launch_step_learned(static_cast<float *>(c->g), make_args<float>(c, t, slot), L, odd, stats, c->grid,
                                     c->stream);
         } else if (c->p.precision == FLBM_FP64)
-            e = launch_step_f64(static_cast<double *>(c->g), make_args<double>(c, t), c->p.scheme, odd,
+            e = launch_step_f64(static_cast<double *>(c->g), make_args<double>(c, t, slot), c->p.scheme, odd,
                                 stats, c->grid, c->row_grid, c->stream);
         else if (c->p.precision == FLBM_FP32)
-            e = launch_step_f32(static_cast<float *>(c->g), make_args<float>(c, t), c->p.scheme, odd,
+            e = launch_step_f32(static_cast<float *>(c->g), make_args<float>(c, t, slot), c->p.scheme, odd,
                                 stats, c->grid, c->row_grid, c->stream);
         else
-            e = launch_step_f16(c->g, make_args<float>(c, t), c->p.scheme, odd, stats, c->grid,
+            e = launch_step_f16(c->g, make_args<float>(c, t, slot), c->p.scheme, odd, stats, c->grid,
                                 c->row_grid, c->stream);
-        if (e != cudaSuccess) return fail(c, FLBM_E_CUDA, std::string("step launch: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            form_totals();   // of the steps that did run
+            return fail(c, FLBM_E_CUDA, std::string("step launch: ") + cudaGetErrorString(e));
+        }
         if (c->timing) {
             CK(c, cudaEventRecord(c->ev[2 * c->ev_used + 1], c->stream));
             ++c->ev_used;
         }
         if (stats) {
-            e = launch_stats_finalize(c->partials, reduced_grid, c->dstats, t, double(c->n), c->stream);
-            if (e != cudaSuccess) return fail(c, FLBM_E_CUDA, std::string("stats launch: ") + cudaGetErrorString(e));
+            f.nblocks[held] = reduced_grid;
+            f.step[held] = t;
+            if (++held == c->stat_slots)
+                if (const int rc = form_totals()) return rc;
         }
     }
+    if (const int rc = form_totals()) return rc;
     c->step += n;
     DevFlags h;
     CK(c, cudaMemcpyAsync(&h, c->dflags, sizeof(h), cudaMemcpyDeviceToHost, c->stream));

@@ -14,7 +14,7 @@ namespace flbm {
 
 struct DevFlags {
     unsigned int flag;
-    unsigned int pad;
+    unsigned int arrived;          // CTAs of the totals' kernel that finished (0 between launches)
     unsigned long long bad_step;
 };
 
@@ -36,7 +36,9 @@ struct flbm_ctx {
     uint32_t tx_pad = 0;           // failure injection into the row pipeline (tests)
     int grid = 1;                  // persistent grid of the direct step kernel
     int row_grid = 0;              // persistent grid of the TMA row pipeline (0: unused)
-    double *partials = nullptr;    // [max(grid, row_grid)][NSTAT]
+    double *partials = nullptr;    // [stat_slots][max_grid][NSTAT], then totals [stat_slots][NSTAT]
+    int stat_slots = 0;            // reduced steps whose partials are kept until their totals are formed
+    int max_grid = 1;              // CTAs of the largest reducing launch
     flbm::DevStats *dstats = nullptr;
     flbm::DevFlags *dflags = nullptr;
     // host transfers: two staging buffers of pipe_nodes * 27 doubles, a copy
@@ -81,7 +83,10 @@ namespace flbm {
 // Parameter check shared by every creation path ("" when valid).
 std::string validate_params(const flbm_params *p);
 // Context creation / destruction (capi.cu).
-int create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void *stream, flbm_ctx **out);
+// stat_slots: steps whose partial sums a context can hold at once (1 to
+// kStatSlots; an ensemble replica is never stepped on its own and takes 1).
+int create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void *stream, flbm_ctx **out,
+               int stat_slots = kStatSlots);
 void destroy_ctx(flbm_ctx *c);
 // A replica's state was replaced: clear the ensemble's sticky failure flags
 // (ensemble.cu).

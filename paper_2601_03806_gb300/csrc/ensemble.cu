@@ -387,7 +387,7 @@ int flbm_ensemble_create(const flbm_params *params, int count, void *cuda_stream
         flbm_ctx *c = nullptr;
         char *slice = static_cast<char *>(e->g) + e->offsets[r];
         const size_t bytes = size_t(params[r].nx) * params[r].ny * params[r].nz * kQ * es;
-        const int rc = create_ctx(&params[r], slice, bytes, e->stream, &c);
+        const int rc = create_ctx(&params[r], slice, bytes, e->stream, &c, 1);
         if (rc != FLBM_OK) {
             e->err = "replica " + std::to_string(r) + ": " + flbm_last_error(nullptr);
             return bail(rc);

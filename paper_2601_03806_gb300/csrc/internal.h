@@ -244,7 +244,16 @@ cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs
                               cudaStream_t s);
 cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, double *S,
                           unsigned long long *cnt, cudaStream_t s);
-cudaError_t launch_stats_finalize(const double *partials, int nblocks, DevStats *st,
-                                  long long step, double n, cudaStream_t s);
+// Partial sums of up to kStatSlots reduced steps, waiting for their totals.
+constexpr int kStatSlots = 16;
+struct StatBatch {
+    const double *partials;        // slot i: [nblocks[i]][NSTAT] at i * slot_stride
+    size_t slot_stride;            // doubles
+    double *totals;                // [kStatSlots][NSTAT] workspace
+    unsigned int *arrived;         // 0 between launches
+    int nblocks[kStatSlots];
+    long long step[kStatSlots];
+};
+cudaError_t launch_stats_finalize(const StatBatch &f, int slots, DevStats *st, double n, cudaStream_t s);
 
 }  // namespace flbm

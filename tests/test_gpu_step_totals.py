@@ -1,4 +1,5 @@
-"""The training pairs, where their code branches."""
+"""Totals of the reduced steps (formed 16 steps at a time), and the
+training pairs, where their code branches."""
 import numpy as np
 import pytest
 
@@ -9,6 +10,35 @@ pytestmark = pytest.mark.gpu
 def F():
     from paper_2601_03806_gb300 import flbm
     return flbm
+
+
+@pytest.mark.parametrize("every", [1, 3])
+@pytest.mark.parametrize("prec,shape", [("fp32", (64, 6, 5)), ("fp64", (5, 4, 3)), ("fp16", (256, 3, 2))])
+def test_totals_do_not_depend_on_how_steps_are_called(F, every, prec, shape):
+    """37 steps in one call, one by one, and 16 + 20 + 1: the same sums."""
+    got = []
+    for calls in ([37], [1] * 37, [16, 20, 1]):
+        box = F.Lattice(*shape, 0.8, 1e-4, seed=2, precision=prec, stats_every=every)
+        box.init_thermal(7)
+        for n in calls:
+            box.step(n)
+        got.append(box.stats())
+    assert got[0]["n_samples"] == (37 if every == 1 else 13)
+    assert got[0]["step"] == 36
+    assert got[0] == got[1] == got[2]
+
+
+def test_moment_state_totals(F):
+    """The first step's totals come from another kernel and grid."""
+    a = F.Lattice(64, 20, 33, 0.8, 1e-4, seed=2, state_form="moments")
+    b = F.Lattice(64, 20, 33, 0.8, 1e-4, seed=2)
+    for box in (a, b):
+        box.init_thermal(7)
+        box.step(19)
+    sa, sb = a.stats(), b.stats()
+    assert sa["n_samples"] == sb["n_samples"] == 19
+    assert np.allclose(sa["u2_avg"], sb["u2_avg"], rtol=1e-5)
+    assert np.allclose(sa["m_var"], sb["m_var"], rtol=1e-4)
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp16", "fp64"])
