@@ -4,7 +4,9 @@
 // reductions.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <type_traits>
 
 #include "internal.h"
@@ -19,6 +21,13 @@ namespace {
 __device__ __forceinline__ void node_xyz(uint64_t n, const BoxDesc &b, uint32_t &x, uint32_t &y,
                                          uint32_t &z)
 {
+    if (b.n <= 0xffffffffull) {   // 32-bit divisions
+        const uint32_t m = uint32_t(n), r = m / b.nx;
+        x = m - r * b.nx;
+        z = r / b.ny;
+        y = r - z * b.ny;
+        return;
+    }
     x = uint32_t(n % b.nx);
     const uint64_t r = n / b.nx;
     y = uint32_t(r % b.ny);
@@ -246,78 +255,255 @@ __global__ void k_moments(const S *g, BoxDesc b, uint64_t n0, uint64_t cn, doubl
     }
 }
 
+// Weight of velocity (cx, cy, cz) in observable OBS (flbm_observable).
+template <int OBS>
+__device__ __forceinline__ constexpr int obs_weight(int cx, int cy, int cz)
+{
+    return OBS == 0   ? 1
+           : OBS == 1 ? cx + cy + cz
+           : OBS == 2 ? cx * cx + cy * cy + cz * cz
+           : OBS == 3 ? cx * cy + cx * cz + cy * cz
+           : OBS == 4 ? cx
+           : OBS == 5 ? cy
+                      : cz;
+}
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+// V consecutive storage elements (one 16-byte load for V > 1) as Acc<S>.
+template <typename S, int V>
+__device__ __forceinline__ void load_vec(const S *p, Acc<S> (&v)[V])
+{
+    if constexpr (V == 1) {
+        v[0] = lda(p, 0);
+    } else {
+        const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(p));
+        S e[V];
+        memcpy(e, &raw, sizeof(raw));
+#pragma unroll
+        for (int q = 0; q < V; ++q) v[q] = lda(e, q);
+    }
+}
+
 // Observable field m(x) (deviation from the rest state; the constant offset
-// only affects the excluded n = 0 mode).
-template <typename S, typename F>
-__global__ void k_observable(const S *g, BoxDesc b, int obs, F *field)
+// only affects the excluded n = 0 mode) and the largest |m|, as the bits of a
+// float, into *peak.  HBM-bound: it reads the 18 to 27 slabs its weights
+// touch.  The observable is a template argument, so every load of a node is
+// issued before the first is used; as a run-time switch inside the loop each
+// waited for the one before (256^3: 854 us, a quarter of the copy rate).  In
+// the natural form nodes are taken V at a time (one 16-byte load per slab,
+// V = 16 / element size); the AA-shifted form shifts them along x, so one at
+// a time (V = 1).
+template <typename S, typename F, int OBS, int V>
+__global__ void __launch_bounds__(256) k_observable(const S *__restrict__ g, const BoxDesc b, F *__restrict__ field,
+                                                    unsigned int *peak)
 {
     using A = Acc<S>;
-    for (uint64_t n = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; n < b.n;
-         n += uint64_t(gridDim.x) * blockDim.x) {
-        uint32_t x, y, z;
-        node_xyz(n, b, x, y, z);
-        A acc = 0;
+    float top = 0.0f;
+    const uint64_t groups = b.n / V;
+    for (uint64_t q = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; q < groups;
+         q += uint64_t(gridDim.x) * blockDim.x) {
+        const uint64_t n = q * V;
+        uint32_t x = 0, y = 0, z = 0;
+        if (V == 1) node_xyz(n, b, x, y, z);
+        A acc[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[e] = 0;
 #pragma unroll
         for (int cx = -1; cx <= 1; ++cx)
 #pragma unroll
             for (int cy = -1; cy <= 1; ++cy)
 #pragma unroll
                 for (int cz = -1; cz <= 1; ++cz) {
-                    int c;
-                    switch (obs) {
-                    case 0: c = 1; break;
-                    case 1: c = cx + cy + cz; break;
-                    case 2: c = cx * cx + cy * cy + cz * cz; break;
-                    case 3: c = cx * cy + cx * cz + cy * cz; break;
-                    case 4: c = cx; break;
-                    case 5: c = cy; break;
-                    default: c = cz; break;
-                    }
-                    if (c != 0) acc += A(c) * lda(g, storage_index(cx, cy, cz, x, y, z, b));
+                    constexpr int zero = 0;
+                    const int c = obs_weight<OBS>(cx, cy, cz);
+                    if (c == zero) continue;
+                    A v[V];
+                    load_vec<S, V>(g + (V == 1 ? storage_index(cx, cy, cz, x, y, z, b)
+                                               : uint64_t(slot_of(cx, cy, cz)) * b.ns + n),
+                                   v);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[e] = fma_(A(c), v[e], acc[e]);
                 }
-        field[n] = F(acc);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            field[n + e] = F(acc[e]);
+            top = fmaxf(top, fabsf(float(acc[e])));
+        }
     }
+    // non-negative floats compare as their bits
+    const unsigned int bits = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+    if ((threadIdx.x & 31) == 0 && bits) atomicMax(peak, bits);
 }
 
+// ---------------------------------------------------------------------------
 // Shell binning of the R2C spectrum [nz][ny][nx/2+1] (complex of T).
-template <typename T>
-__global__ void k_shells(const T *spec, BoxDesc b, int nshell, double *S, unsigned long long *cnt)
+
+// A sum of squares: FP32 spectra keep it as an exact-to-48-bits FP32 pair
+// (FP64 operations, two per clock and SM, bounded the kernel before: 84 % of
+// that pipe, 324 us at 256^3), FP64 spectra in FP64.
+template <typename T> struct ShellSum;
+template <> struct ShellSum<float> {
+    float hi, lo;
+    __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
+    __device__ __forceinline__ void add(float h, float l)
+    {
+        float e;
+        hi = two_sum(hi, h, e);
+        lo += e + l;
+    }
+    __device__ __forceinline__ void add(const ShellSum &o) { add(o.hi, o.lo); }
+    __device__ __forceinline__ void add_square(float v)
+    {
+        const float p = __fmul_rn(v, v);
+        add(p, __fmaf_rn(v, v, -p));
+    }
+    __device__ __forceinline__ void scale2() { hi *= 2.0f; lo *= 2.0f; }
+    __device__ __forceinline__ ShellSum up(int d) const
+    {
+        return ShellSum{__shfl_up_sync(0xffffffffu, hi, d), __shfl_up_sync(0xffffffffu, lo, d)};
+    }
+    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
+};
+template <> struct ShellSum<double> {
+    double v;
+    __device__ __forceinline__ void zero() { v = 0.0; }
+    __device__ __forceinline__ void add(const ShellSum &o) { v += o.v; }
+    __device__ __forceinline__ void add_square(double x) { v = fma(x, x, v); }
+    __device__ __forceinline__ void scale2() { v *= 2.0; }
+    __device__ __forceinline__ ShellSum up(int d) const { return ShellSum{__shfl_up_sync(0xffffffffu, v, d)}; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+// Power of two that brings a spectrum whose field peaks at `peak` into a
+// range where FP32 squares neither overflow nor underflow: every amplitude is
+// at most N peak, and so is the root of the sum of all squares (Parseval);
+// N peak goes to about 2^60.  Exact, and divided out of the totals.
+__device__ __forceinline__ float shell_scale(unsigned int peak_bits, uint64_t n)
 {
-    extern __shared__ double smem[];
-    double *sh_s = smem;
-    unsigned long long *sh_c = reinterpret_cast<unsigned long long *>(smem + nshell);
-    for (int s = threadIdx.x; s < nshell; s += blockDim.x) { sh_s[s] = 0.0; sh_c[s] = 0ull; }
-    __syncthreads();
-    const uint32_t nxh = b.nx / 2 + 1;
-    const uint64_t total = uint64_t(nxh) * b.ny * b.nz;
-    const double invN = 1.0 / double(b.n);
-    for (uint64_t e = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; e < total;
-         e += uint64_t(gridDim.x) * blockDim.x) {
-        const uint32_t kx = uint32_t(e % nxh);
-        const uint64_t r = e / nxh;
-        const uint32_t ky = uint32_t(r % b.ny), kz = uint32_t(r / b.ny);
-        const long long ax = kx;
-        const long long ay = (2ull * ky < b.ny) ? (long long)ky : (long long)ky - (long long)b.ny;
-        const long long az = (2ull * kz < b.nz) ? (long long)kz : (long long)kz - (long long)b.nz;
-        const long long n2 = ax * ax + ay * ay + az * az;
-        if (n2 == 0) continue;
-        // round(|n|): s^2 - s < n2 <= s^2 + s for integer s (|n| is never a half-integer)
-        long long s = llrint(sqrt(double(n2)));
-        while (s * s - s >= n2) --s;
-        while (s * s + s < n2) ++s;
-        if (s >= nshell) continue;
-        const double re = double(spec[2 * e]), im = double(spec[2 * e + 1]);
-        // the conjugate half (kx -> -kx) has the same |n|; kx = 0 and the even
-        // Nyquist plane are their own partners
-        const unsigned wgt = (kx == 0 || (b.nx % 2 == 0 && kx == b.nx / 2)) ? 1u : 2u;
-        atomicAdd(&sh_s[s], wgt * (re * re + im * im) * invN);
-        atomicAdd(&sh_c[s], (unsigned long long)wgt);
+    const float peak = __uint_as_float(peak_bits);
+    if (!(peak > 0.0f) || !(peak < INFINITY)) return 1.0f;
+    int k = 60 - (ilogb(double(peak)) + 1) - (64 - __clzll((long long)n));
+    k = k > 126 ? 126 : (k < -126 ? -126 : k);
+    return __uint_as_float(uint32_t(127 + k) << 23);
+}
+
+// round(|n|) of n2 = |n|^2: 0, or the s >= 1 with s^2 - s < n2 <= s^2 + s (|n|
+// is never a half-integer), from a square root good to one.
+__device__ __forceinline__ long long shell_of(unsigned long long n2)
+{
+    if (n2 == 0) return 0;
+    long long s = n2 < (1ull << 44) ? (long long)(__fsqrt_rn(float(n2)) + 0.5f) : llrint(sqrt(double(n2)));
+    while (s * s - s >= (long long)n2) --s;
+    while (s * s + s < (long long)n2) ++s;
+    return s;
+}
+
+constexpr int kShellWarps = 8;
+constexpr size_t kShellSmem = 200 * 1024;
+// Warps of a CTA whose private bins (a sum and a count per shell) fit.
+inline int shell_warps(int nshell)
+{
+    const size_t w = kShellSmem / (size_t(nshell) * (sizeof(double) + sizeof(unsigned int)));
+    return w < size_t(kShellWarps) ? int(w) : kShellWarps;
+}
+
+// A warp takes the rows kx = 0 .. nx/2 of (+-ky, +-kz), up to four at once:
+// they have the same |n| element by element, so one shell index and one
+// binning serve four values.  Along a row the shell only grows, so lanes of
+// one shell are neighbours: a segmented scan leaves each shell's sum on its
+// last lane, which adds it to the warp's own bins in shared memory -- no
+// atomics until the CTA's totals, added in FP64.  Rows stop at the last
+// shell asked for.
+template <typename T>
+__global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict__ spec, const BoxDesc b, int nshell,
+                                                             const unsigned int *peak, double *S,
+                                                             unsigned long long *cnt)
+{
+    extern __shared__ __align__(16) unsigned char shell_raw[];
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ShellSum<T> *const sums = reinterpret_cast<ShellSum<T> *>(shell_raw);
+    unsigned int *const cnts = reinterpret_cast<unsigned int *>(shell_raw + size_t(warps) * nshell * sizeof(double));
+    static_assert(sizeof(ShellSum<T>) == sizeof(double), "a bin is 8 bytes");
+    for (int i = threadIdx.x; i < warps * nshell; i += blockDim.x) {
+        sums[i].zero();
+        cnts[i] = 0u;
     }
     __syncthreads();
+    ShellSum<T> *const bin = sums + size_t(warp) * nshell;
+    unsigned int *const num = cnts + size_t(warp) * nshell;
+    const uint32_t nxh = b.nx / 2 + 1, nyh = b.ny / 2 + 1, nzh = b.nz / 2 + 1;
+    const float scale = std::is_same<T, float>::value ? shell_scale(*peak, b.n) : 1.0f;
+    const uint64_t rows = uint64_t(nyh) * nzh;
+    for (uint64_t r = blockIdx.x * uint64_t(warps) + warp; r < rows; r += uint64_t(gridDim.x) * warps) {
+        const uint32_t ay = uint32_t(r % nyh), az = uint32_t(r / nyh);
+        const bool two_y = ay != 0 && 2 * uint64_t(ay) != b.ny, two_z = az != 0 && 2 * uint64_t(az) != b.nz;
+        const unsigned long long perp = (unsigned long long)ay * ay + (unsigned long long)az * az;
+        const int mult = (two_y ? 2 : 1) * (two_z ? 2 : 1);
+        const T *row[4];   // (ky, kz), (-ky, kz), (ky, -kz), (-ky, -kz)
+        row[0] = spec + 2 * (uint64_t(az) * b.ny + ay) * nxh;
+        row[1] = spec + 2 * (uint64_t(az) * b.ny + (b.ny - ay)) * nxh;
+        row[2] = spec + 2 * (uint64_t(b.nz - az) * b.ny + ay) * nxh;
+        row[3] = spec + 2 * (uint64_t(b.nz - az) * b.ny + (b.ny - ay)) * nxh;
+        for (uint32_t k0 = 0; k0 < nxh; k0 += 32) {
+            const uint32_t kx = k0 + lane;
+            const long long s = shell_of((unsigned long long)kx * kx + perp);
+            const bool in = kx < nxh && s < nshell;
+            // lanes of one row: in holds on a prefix of the warp
+            const unsigned int on = __ballot_sync(0xffffffffu, in);
+            if (!on) break;
+            // the conjugate half (kx -> -kx) has the same |n|; kx = 0 and the
+            // even Nyquist plane are their own partners
+            const bool own = kx == 0 || (b.nx % 2 == 0 && kx == b.nx / 2);
+            ShellSum<T> v;
+            v.zero();
+            if (in) {
+                T re[4], im[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool use = (!(q & 1) || two_y) && (!(q & 2) || two_z);
+                    re[q] = use ? row[q][2 * kx] * T(scale) : T(0);
+                    im[q] = use ? row[q][2 * kx + 1] * T(scale) : T(0);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    v.add_square(re[q]);
+                    v.add_square(im[q]);
+                }
+                if (!own) v.scale2();
+            }
+            const int sh = in ? int(s) : -1;
+            const int left = __shfl_up_sync(0xffffffffu, sh, 1);
+            const unsigned int heads = __ballot_sync(0xffffffffu, in && (lane == 0 || left != sh));
+            const unsigned int owns = __ballot_sync(0xffffffffu, in && own);
+            const unsigned int upto = 0xffffffffu >> (31 - lane);        // lanes 0 .. lane
+            const int head = in ? 31 - __clz(int(heads & upto)) : lane;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const ShellSum<T> o = v.up(d);
+                if (lane - d >= head) v.add(o);
+            }
+            const bool tail = in && (lane == 31 || (((heads | ~on) >> (lane + 1)) & 1u));
+            if (tail && sh > 0) {   // shell 0 holds only n = 0, which is excluded
+                const unsigned int seg = upto & ~((1u << head) - 1u);
+                bin[sh].add(v);
+                num[sh] += unsigned(mult) * (2u * __popc(seg) - __popc(owns & seg));
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    const double inv = 1.0 / (double(b.n) * double(scale) * double(scale));
     for (int s = threadIdx.x; s < nshell; s += blockDim.x) {
-        if (sh_c[s]) {
-            atomicAdd(&S[s], sh_s[s]);
-            atomicAdd(&cnt[s], sh_c[s]);
+        double t = 0.0;
+        unsigned long long k = 0;
+        for (int w = 0; w < warps; ++w) {
+            t += sums[size_t(w) * nshell + s].value();
+            k += cnts[size_t(w) * nshell + s];
+        }
+        if (k) {
+            atomicAdd(&S[s], t * inv);
+            atomicAdd(&cnt[s], k);
         }
     }
 }
@@ -602,30 +788,57 @@ cudaError_t launch_moments(const void *g, int prec, const BoxDesc &b, uint64_t n
     return cudaGetLastError();
 }
 
+namespace {
+template <typename S, int V>
+void observable(const void *g, const BoxDesc &b, int obs, void *field, unsigned int *peak, int grid, cudaStream_t s)
+{
+    using F = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
+    const S *p = static_cast<const S *>(g);
+    F *f = static_cast<F *>(field);
+    switch (obs) {
+    case 0: k_observable<S, F, 0, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    case 1: k_observable<S, F, 1, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    case 2: k_observable<S, F, 2, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    case 3: k_observable<S, F, 3, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    case 4: k_observable<S, F, 4, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    case 5: k_observable<S, F, 5, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    default: k_observable<S, F, 6, V><<<grid, 256, 0, s>>>(p, b, f, peak); break;
+    }
+}
+}  // namespace
+
 // The observable field is double for FP64 storage and float otherwise.
-cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs, void *field,
+cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs, void *field, unsigned int *peak,
                               cudaStream_t s)
 {
-    const int grid = grid_for(b.n, 256);
     with_storage(prec, [&](auto tag) {
         using S = decltype(tag);
-        using F = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
-        k_observable<S, F><<<grid, 256, 0, s>>>(static_cast<const S *>(g), b, obs, static_cast<F *>(field));
+        constexpr int V = 16 / int(sizeof(S));
+        // 16-byte loads: natural form, whole groups of V, every slab (256-byte
+        // aligned buffer) starting on 16 bytes
+        const bool vec = b.parity == 0 && b.n % V == 0 && b.ns % V == 0;
+        const uint64_t groups = vec ? b.n / V : b.n;
+        const int grid = int(std::min<uint64_t>((groups + 255) / 256, 152 * 16));
+        if (vec) observable<S, V>(g, b, obs, field, peak, grid, s);
+        else observable<S, 1>(g, b, obs, field, peak, grid, s);
     });
     return cudaGetLastError();
 }
 
-cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, double *S,
+cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, const unsigned int *peak, double *S,
                           unsigned long long *cnt, cudaStream_t s)
 {
-    const uint64_t total = uint64_t(b.nx / 2 + 1) * b.ny * b.nz;
-    int grid = grid_for(total, 256);
-    if (grid > 2048) grid = 2048;
-    const size_t sm = size_t(nshell) * (sizeof(double) + sizeof(unsigned long long));
-    if (prec == 0)
-        k_shells<double><<<grid, 256, sm, s>>>(static_cast<const double *>(spec), b, nshell, S, cnt);
-    else
-        k_shells<float><<<grid, 256, sm, s>>>(static_cast<const float *>(spec), b, nshell, S, cnt);
+    const int warps = shell_warps(nshell);
+    const uint64_t rows = uint64_t(b.ny / 2 + 1) * (b.nz / 2 + 1);
+    const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, 152 * 4));
+    const size_t sm = size_t(warps) * nshell * (sizeof(double) + sizeof(unsigned int));
+    if (prec == 0) {
+        cudaFuncSetAttribute(k_shells<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
+        k_shells<double><<<grid, 32 * warps, sm, s>>>(static_cast<const double *>(spec), b, nshell, peak, S, cnt);
+    } else {
+        cudaFuncSetAttribute(k_shells<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
+        k_shells<float><<<grid, 32 * warps, sm, s>>>(static_cast<const float *>(spec), b, nshell, peak, S, cnt);
+    }
     return cudaGetLastError();
 }
 

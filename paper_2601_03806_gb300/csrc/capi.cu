@@ -303,7 +303,6 @@ void flbm::destroy_ctx(flbm_ctx *c)
     cudaFree(c->fft_in);
     cudaFree(c->fft_out);
     cudaFree(c->shell_s);
-    cudaFree(c->shell_c);
     if (c->copy_stream) cudaStreamSynchronize(c->copy_stream);
     for (int b = 0; b < 2; ++b) {
         cudaFree(c->pipe[b]);
@@ -680,29 +679,29 @@ int flbm_structure_factor(flbm_ctx *c, int observable, int nshell, double *S, in
         c->has_plan = true;
     }
     CKFFT(c, cufftSetStream(c->plan, c->stream));
+    // one workspace: S, counts, the field's peak
+    const size_t shell_bytes = nshell * (sizeof(double) + sizeof(unsigned long long)) + sizeof(unsigned int);
     if (nshell > c->shell_cap) {
         cudaFree(c->shell_s);
-        cudaFree(c->shell_c);
         c->shell_s = nullptr;
-        c->shell_c = nullptr;
         c->shell_cap = 0;
-        CK(c, cudaMalloc(&c->shell_s, nshell * sizeof(double)));
-        CK(c, cudaMalloc(&c->shell_c, nshell * sizeof(unsigned long long)));
+        CK(c, cudaMalloc(&c->shell_s, shell_bytes));
         c->shell_cap = nshell;
     }
+    unsigned long long *const shell_c = reinterpret_cast<unsigned long long *>(c->shell_s + nshell);
+    unsigned int *const peak = reinterpret_cast<unsigned int *>(shell_c + nshell);
+    CK(c, cudaMemsetAsync(c->shell_s, 0, shell_bytes, c->stream));
     const BoxDesc b = box_of(c);
-    CK(c, launch_observable(c->g, prec_code(c), b, observable, c->fft_in, c->stream));
+    CK(c, launch_observable(c->g, prec_code(c), b, observable, c->fft_in, peak, c->stream));
     if (dbl)
         CKFFT(c, cufftExecD2Z(c->plan, static_cast<cufftDoubleReal *>(c->fft_in),
                               static_cast<cufftDoubleComplex *>(c->fft_out)));
     else
         CKFFT(c, cufftExecR2C(c->plan, static_cast<cufftReal *>(c->fft_in),
                               static_cast<cufftComplex *>(c->fft_out)));
-    CK(c, cudaMemsetAsync(c->shell_s, 0, nshell * sizeof(double), c->stream));
-    CK(c, cudaMemsetAsync(c->shell_c, 0, nshell * sizeof(unsigned long long), c->stream));
-    CK(c, launch_shells(c->fft_out, prec_code(c), b, nshell, c->shell_s, c->shell_c, c->stream));
+    CK(c, launch_shells(c->fft_out, prec_code(c), b, nshell, peak, c->shell_s, shell_c, c->stream));
     CK(c, cudaMemcpyAsync(S, c->shell_s, nshell * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(c, cudaMemcpyAsync(count, c->shell_c, nshell * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaMemcpyAsync(count, shell_c, nshell * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     for (int s = 0; s < nshell; ++s)
         if (count[s] > 0) S[s] /= double(count[s]);

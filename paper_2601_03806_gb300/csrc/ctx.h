@@ -53,8 +53,7 @@ struct flbm_ctx {
     bool has_plan = false;
     void *fft_in = nullptr;
     void *fft_out = nullptr;
-    double *shell_s = nullptr;
-    unsigned long long *shell_c = nullptr;
+    double *shell_s = nullptr;     // S, counts and the field's peak of up to shell_cap shells
     int shell_cap = 0;
     // step-kernel timing
     bool timing = false;

@@ -240,9 +240,11 @@ cudaError_t launch_probe(const void *g, int prec, const BoxDesc &b, const long l
                          long long count, double *out, cudaStream_t s);
 cudaError_t launch_moments(const void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,
                            double *out, cudaStream_t s);
-cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs, void *field,
+// *peak (0 before): the bits of the field's largest magnitude, which
+// launch_shells takes.
+cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs, void *field, unsigned int *peak,
                               cudaStream_t s);
-cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, double *S,
+cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, const unsigned int *peak, double *S,
                           unsigned long long *cnt, cudaStream_t s);
 // Partial sums of up to kStatSlots reduced steps, waiting for their totals.
 constexpr int kStatSlots = 16;
