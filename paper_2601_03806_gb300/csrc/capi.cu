@@ -19,6 +19,7 @@
 #include "ctx.h"
 #include "internal.h"
 #include "lattice.cuh"
+#include "normal_tab_host.h"
 
 using namespace flbm;
 
@@ -74,6 +75,17 @@ uint64_t slab_stride(uint64_t n, size_t es)
         if (v >= 0 && v % 128 == 0 && v <= (1ll << 30)) pad = uint64_t(v);
     }
     return (n + 63) / 64 * 64 + pad / es;
+}
+
+// The FP64 Box-Muller tables, formed once per process.
+const NormalTab &normal_tab()
+{
+    static const NormalTab *const t = [] {
+        NormalTab *p = new NormalTab;
+        build_normal_tab(*p);
+        return p;
+    }();
+    return *t;
 }
 
 int prec_code(const flbm_ctx *c) { return c->p.precision == FLBM_FP64 ? 0 : (c->p.precision == FLBM_FP32 ? 1 : 2); }
@@ -200,6 +212,7 @@ StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr)
     a.step = uint64_t(t);
     fill_constants_t<R>(c->p, a);
     a.tx_pad = c->tx_pad;
+    a.normals = c->normals;
     a.partials = partials;
     a.flag = &c->dflags->flag;
     a.bad_step = &c->dflags->bad_step;
@@ -315,6 +328,7 @@ void flbm::destroy_ctx(flbm_ctx *c)
     cudaFree(c->dflags);
     if (c->own_g) cudaFree(c->g);
     cudaFree(c->mlp_img);
+    cudaFree(c->normals);
     cudaFree(c->ms[0]);
     cudaFree(c->ms[1]);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -411,6 +425,13 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
     if (e == cudaSuccess) e = cudaMalloc(&c->dstats, sizeof(DevStats));
     if (e == cudaSuccess) e = cudaMalloc(&c->dflags, sizeof(DevFlags));
     if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_NOMEM); }
+    if (p->precision == FLBM_FP64) {
+        const NormalTab &tab = normal_tab();
+        e = cudaMalloc(&c->normals, sizeof(tab));
+        if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_NOMEM); }
+        e = cudaMemcpyAsync(c->normals, &tab, sizeof(tab), cudaMemcpyHostToDevice, c->stream);
+        if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_CUDA); }
+    }
     e = cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream);
     if (e == cudaSuccess) e = launch_fill_rest(c->g, prec_code(c), c->ns * kQ, c->stream);
     if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return bail(FLBM_E_CUDA); }

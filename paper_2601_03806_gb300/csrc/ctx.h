@@ -48,6 +48,7 @@ struct flbm_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_ready[2] = {nullptr, nullptr};
     cudaEvent_t ev_free[2] = {nullptr, nullptr};
+    flbm::NormalTab *normals = nullptr;   // FP64: tables of the Box-Muller transform
     // S(k)
     cufftHandle plan = 0;
     bool has_plan = false;

@@ -8,6 +8,8 @@ struct flbm_params;
 
 namespace flbm {
 
+struct NormalTab;   // normal_tab.cuh
+
 constexpr int kQ = 27;
 constexpr int NSTAT = 13;     // fused reduction slots, see StatSlot
 constexpr int kBlock = 128;   // threads per CTA of the step kernel (one x-row chunk)
@@ -51,6 +53,7 @@ struct StepArgs {
     R omega;                      // weight of the equilibrium in k = 4..9
     R amp_h;                      // sqrt(kT omega (2 - omega)), Eq. fluct_phi
     R amp_g;                      // ghosts: sqrt(kT) (Eq. fluct_phig), amp_h for BGK
+    const NormalTab *normals;     // FP64: the tables of the Box-Muller transform
     double *partials;             // [gridDim.x][NSTAT] when reducing
     unsigned int *flag;           // bit 0: instability; bit 1: a bounded wait ran out
     unsigned long long *bad_step; // first step that met rho <= 0 / non-finite

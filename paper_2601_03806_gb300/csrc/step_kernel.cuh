@@ -53,6 +53,7 @@
 
 #include "internal.h"
 #include "lattice.cuh"
+#include "normal_tab.cuh"
 
 namespace flbm {
 
@@ -346,15 +347,14 @@ __device__ __forceinline__ void normal_pair(uint32_t w1, uint32_t w2, float &rad
     rad = __fmul_rn(t, rsqrtf(t));
     __sincosf(__fmaf_rn(u2, 6.2831853071795865f, -3.1415926535897932f), &sa, &ca);
 }
-__device__ __forceinline__ void normal_pair(uint32_t w1, uint32_t w2, double &rad, double &ca, double &sa)
+// FP64: from tables (normal_tab.cuh), 32 FP64 operations a pair instead of
+// about 75 with the library's log and sincospi; the FP64 pipe bounds the
+// FP64 step (86 % busy; 1350 operations a node before).
+__device__ __forceinline__ void normal_pair(const NormalTab &tab, uint32_t w1, uint32_t w2, double &rad, double &ca,
+                                            double &sa)
 {
-    const double u1 = uniform23d(w1);
-    const double u2 = uniform23d(w2);
-    rad = sqrt(-2.0 * log(u1));
-    double s, c;
-    sincospi(2.0 * u2, &s, &c);
-    ca = -c;
-    sa = -s;
+    rad = sqrt(neg2_log(tab, w1 >> 9));
+    neg_cos_sin(tab, w2 >> 9, ca, sa);
 }
 // Two nodes, one per lane (words of node a in .x, of node b in .y).
 __device__ __forceinline__ void normal_pair(uint2 w1, uint2 w2, float2 &rad, float2 &ca, float2 &sa)
@@ -384,6 +384,10 @@ __device__ __forceinline__ void block_normals(const A &a, uint32_t node, int blk
         const u32x4 oa = noise_block(a, node, blk), ob = noise_block(a, node + 1, blk);
         normal_pair(make_uint2(oa.x, ob.x), make_uint2(oa.y, ob.y), rad0, c0, s0);
         normal_pair(make_uint2(oa.z, ob.z), make_uint2(oa.w, ob.w), rad1, c1, s1);
+    } else if constexpr (std::is_same<V, double>::value) {
+        const u32x4 o = noise_block(a, node, blk);
+        normal_pair(*a.normals, o.x, o.y, rad0, c0, s0);
+        normal_pair(*a.normals, o.z, o.w, rad1, c1, s1);
     } else {
         const u32x4 o = noise_block(a, node, blk);
         normal_pair(o.x, o.y, rad0, c0, s0);

@@ -1,5 +1,5 @@
-"""Totals of the reduced steps (formed 16 steps at a time), and the
-training pairs, where their code branches."""
+"""Totals of the reduced steps (formed 16 steps at a time), the FP64 normals
+from tables, and the training pairs, where their code branches."""
 import numpy as np
 import pytest
 
@@ -39,6 +39,20 @@ def test_moment_state_totals(F):
     assert sa["n_samples"] == sb["n_samples"] == 19
     assert np.allclose(sa["u2_avg"], sb["u2_avg"], rtol=1e-5)
     assert np.allclose(sa["m_var"], sb["m_var"], rtol=1e-4)
+
+
+@pytest.mark.parametrize("shape", [(32, 31, 29), (37, 21, 19)])
+def test_fp64_noise_matches_the_oracle(F, oracle_mod, shape):
+    """One step from rest is the noise alone (27,000 nodes, 325,000 pairs of
+    normals, row and direct kernels): a radius and an angle good to 2^-52 and
+    2^-52, 23 terms of size sqrt(3 kT) at most, summed in three passes: 2^-46
+    of that scale."""
+    kT = 1e-2
+    box = F.Lattice(*shape, 1.0, kT, seed=99, precision="fp64")
+    ref = oracle_mod.Box(*shape, 1.0, kT, seed=99)
+    box.step(1)
+    ref.step(1)
+    assert np.abs(box.get_populations() - ref.get_f()).max() <= 2.0 ** -46 * np.sqrt(3 * kT)
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp16", "fp64"])
