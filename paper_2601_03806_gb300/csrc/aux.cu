@@ -646,11 +646,12 @@ __global__ void __launch_bounds__(kPairBlock) k_mlp_pairs(const S *__restrict__ 
 // order, a thread per component.  One launch per kStatSlots steps, and 13
 // CTAs per step because FP64 adds run at two per clock and SM: one CTA per
 // step took 15-17 us a step, a seventh of the 128^3 step and most of the 64^3
-// one; this takes about 5 us per launch.
+// one; with the means' divisions in parallel this takes under 1 us a step.
 constexpr int kStatThreads = 128;
 __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch f, DevStats *st, double n)
 {
-    __shared__ double red[kStatThreads];
+    __shared__ double red[kStatSlots * kStatTerms];   // at least kStatThreads
+    static_assert(kStatSlots * kStatTerms >= kStatThreads, "the sums use it too");
     __shared__ bool last;
     const int s = blockIdx.x, i = blockIdx.y, t = threadIdx.x;
     const double *p = f.partials + size_t(i) * f.slot_stride + s;
@@ -671,7 +672,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch
     __syncthreads();
     if (!last) return;
     __threadfence();
-    stats_update(st, f.totals, int(gridDim.y), f.step, n, t);
+    stats_update(st, f.totals, int(gridDim.y), f.step, n, red);
     if (t == 0) *f.arrived = 0u;
 }
 

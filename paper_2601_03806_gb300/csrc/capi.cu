@@ -394,14 +394,10 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
         c->own_g = true;
     }
     // persistent grids: resident CTAs of the reducing (larger) variants
-    int occ = 1, occ_rows = 0;
-    if (p->precision == FLBM_FP64)
-        step_occupancy_f64(p->scheme, uint32_t(p->nx), true, occ, occ_rows);
-    else if (p->precision == FLBM_FP32)
-        step_occupancy_f32(p->scheme, uint32_t(p->nx), c->ns, true, occ, occ_rows);
-    else
-        step_occupancy_f16(p->scheme, uint32_t(p->nx), c->ns, true, occ, occ_rows);
-    step_grids(*p, c->nsm, occ, occ_rows, c->grid, c->row_grid);
+    const auto step_shape = p->precision == FLBM_FP64   ? step_shape_f64
+                            : p->precision == FLBM_FP32 ? step_shape_f32
+                                                        : step_shape_f16;
+    step_grids(*p, c->nsm, step_shape(p->scheme, uint32_t(p->nx), c->n, c->ns, true), c->grid, c->row_grid);
     // FLBM_INJECT_STARVE=1 (environment, failure-injection tests only): the
     // row pipeline expects 16 bytes more than it copies (the learned step
     // issues no first-layer MMA), so the bounded waits run out and flbm_step
@@ -444,26 +440,29 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
 }
 
 namespace flbm {
-void step_grids(const flbm_params &p, int nsm, int occ, int occ_rows, int &grid, int &row_grid)
+void step_grids(const flbm_params &p, int nsm, const StepShape &shape, int &grid, int &row_grid)
 {
     const uint64_t n = uint64_t(p.nx) * uint64_t(p.ny) * uint64_t(p.nz);
-    const uint64_t nchunks = uint64_t((p.nx + kBlock - 1) / kBlock) * p.ny * p.nz;
+    // the learned step and the moment form's first step take 128-node row
+    // chunks, the direct kernel the shape's CTAs
+    const bool chunks = p.scheme == FLBM_LEARNED || p.state_form == FLBM_STATE_MOMENTS;
+    const uint64_t work = chunks ? uint64_t((p.nx + kBlock - 1) / kBlock) * p.ny * p.nz : shape.ctas;
     // FLBM_CTAS_PER_SM (environment) caps the direct kernel's grid below the
     // occupancy limit; a tuning knob, the default is the occupancy limit
-    int per_sm = occ;
+    int per_sm = chunks ? 4 : shape.direct;
     if (const char *env = std::getenv("FLBM_CTAS_PER_SM")) {
         const int v = std::atoi(env);
-        if (v > 0 && v < occ) per_sm = v;
+        if (v > 0 && v < per_sm) per_sm = v;
     }
     if (p.scheme == FLBM_LEARNED) per_sm = learned_occupancy(n);
-    grid = int(std::min<uint64_t>(nchunks, uint64_t(nsm) * per_sm));
+    grid = int(std::min<uint64_t>(work, uint64_t(nsm) * per_sm));
     if (grid < 1) grid = 1;
     // FLBM_ROWS=0 (environment) disables the TMA row pipeline
     row_grid = 0;
     const char *rows_env = std::getenv("FLBM_ROWS");
-    if (occ_rows > 0 && p.scheme != FLBM_LEARNED && !(rows_env && std::atoi(rows_env) == 0)) {
+    if (shape.rows > 0 && p.scheme != FLBM_LEARNED && !(rows_env && std::atoi(rows_env) == 0)) {
         const uint64_t nrows = uint64_t(p.ny) * p.nz;
-        row_grid = int(std::min<uint64_t>(nrows, uint64_t(nsm) * occ_rows));
+        row_grid = int(std::min<uint64_t>(nrows, uint64_t(nsm) * shape.rows));
     }
 }
 

@@ -151,13 +151,21 @@ cudaError_t launch_step_f32(float *g, const StepArgs<float> &a, int scheme, bool
                             bool stats, int grid, int row_grid, cudaStream_t s);
 cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool odd,
                             bool stats, int grid, int row_grid, cudaStream_t s);
-// Resident CTAs per SM of the direct kernel and of the row pipeline (0 when
-// it does not serve rows of length nx) for (precision, scheme, stats; ns, the
-// slab stride, picks the index width); also
-// prepares the kernels' shared-memory attributes on the current device.
-void step_occupancy_f64(int scheme, uint32_t nx, bool stats, int &direct, int &rows);
-void step_occupancy_f32(int scheme, uint32_t nx, uint64_t ns, bool stats, int &direct, int &rows);
-void step_occupancy_f16(int scheme, uint32_t nx, uint64_t ns, bool stats, int &direct, int &rows);
+// Nodes from which the direct kernel takes two per thread in CTAs of kBlock
+// threads (below, one per thread in CTAs of a warp).
+constexpr uint64_t kDirectPairs = 65536;
+// Launch shape of the step kernels for a box of n nodes in rows of nx: the
+// direct kernel's CTAs and how many of them an SM holds, and the row
+// pipeline's CTAs per SM (0 when it does not serve rows of length nx); the
+// slab stride ns picks the index width.  Also prepares the kernels'
+// shared-memory attributes on the current device.
+struct StepShape {
+    uint64_t ctas = 1;
+    int direct = 1, rows = 0;
+};
+StepShape step_shape_f64(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
+StepShape step_shape_f32(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
+StepShape step_shape_f16(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
 // The FP16-storage two-node row kernels for rows of exactly 512 nodes
 // (step_f16_nx512.cu), which step_f16.cu calls when the row plan of the box
 // takes two nodes per thread in full CTAs.  FP32 keeps the general kernel:
@@ -175,9 +183,9 @@ int rows_occupancy_f32_paced(int scheme, bool stats, uint32_t nx);
 // Philox round keys, the density used by the noise, and the per-mode
 // relaxation / equilibrium / noise coefficients of the scheme.
 // Grids of the direct step kernel and of the row pipeline (0: not used) for
-// a box on nsm SMs, given the kernels' resident CTAs per SM; honours the
+// a box on nsm SMs, given the kernels' launch shape; honours the
 // FLBM_CTAS_PER_SM and FLBM_ROWS=0 environment knobs.
-void step_grids(const flbm_params &p, int nsm, int occ, int occ_rows, int &grid, int &row_grid);
+void step_grids(const flbm_params &p, int nsm, const StepShape &shape, int &grid, int &row_grid);
 void fill_step_constants(const flbm_params &p, StepArgs<float> &a);
 void fill_step_constants(const flbm_params &p, StepArgs<double> &a);
 // Set the calling thread's error text returned by flbm_last_error(NULL).

@@ -157,13 +157,6 @@ struct TileWalk {
     }
 };
 
-__device__ __forceinline__ void cp_async4(float *dst, const float *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
 // Threads kGradThreads - T ..: the sample rows of the tile at w into idx.
 template <int T>
 __device__ __forceinline__ void tile_rows(uint64_t (&idx)[T], const Samples &s, const TileWalk<T> &w)

@@ -19,26 +19,33 @@ __device__ __forceinline__ void stats_update(DevStats *st, const double *red, lo
     st->nsamp += 1;
 }
 
-// The same for `count` consecutive reduced steps, in order: totals[i][NSTAT]
-// of time step[i], a thread t per component (at least 32 threads call it;
-// the loads bypass the L1, other SMs wrote them).
+// The same for `count` <= kStatSlots consecutive reduced steps, in order, by
+// the threads of a CTA: totals[i][NSTAT] of time step[i] (loads bypass the
+// L1: other SMs wrote them).  The means are formed in parallel (FP64
+// divisions one after the other took most of the time), then a thread per
+// accumulator adds them in step order; mean: kStatSlots * kStatTerms doubles
+// of shared memory.
+constexpr int kStatTerms = 11;   // acc_u2, acc_m, acc_m2
 __device__ __forceinline__ void stats_update(DevStats *st, const double *totals, int count, const long long *step,
-                                             double n, int t)
+                                             double n, double *mean)
 {
-    if (t < NSTAT) st->last[t] = __ldcg(totals + (count - 1) * NSTAT + t);
-    if (t < 11) {
-        // accumulator t and the sums it takes
-        double *acc = t < 3 ? &st->acc_u2[t] : (t < 7 ? &st->acc_m[t - 3] : &st->acc_m2[t - 7]);
+    for (int e = threadIdx.x; e < count * kStatTerms; e += blockDim.x) {
+        const int t = e % kStatTerms;
+        const double *r = totals + e / kStatTerms * NSTAT;
         const int slot = t < 3   ? S_UX2 + t
                          : t < 7 ? (t == 3 ? S_DRHO : (t == 4 ? S_JX : (t == 5 ? S_M3 : S_M4)))
                                  : S_M1SQ + t - 7;
+        double v = __ldcg(r + slot);
+        if (t == 4) v = (v + __ldcg(r + S_JY)) + __ldcg(r + S_JZ);
+        mean[e] = v / n;
+    }
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < NSTAT) st->last[t] = __ldcg(totals + (count - 1) * NSTAT + t);
+    if (t < kStatTerms) {
+        double *acc = t < 3 ? &st->acc_u2[t] : (t < 7 ? &st->acc_m[t - 3] : &st->acc_m2[t - 7]);
         double a = *acc;
-        for (int i = 0; i < count; ++i) {
-            const double *r = totals + i * NSTAT;
-            double v = __ldcg(r + slot);
-            if (t == 4) v = (v + __ldcg(r + S_JY)) + __ldcg(r + S_JZ);
-            a += v / n;
-        }
+        for (int i = 0; i < count; ++i) a += mean[i * kStatTerms + t];
         *acc = a;
     }
     if (t == 31) {

@@ -20,11 +20,12 @@ cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool 
     return launch_step_t<__half, float, uint64_t>(h, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-void step_occupancy_f16(int scheme, uint32_t nx, uint64_t ns, bool stats, int &direct, int &rows)
+StepShape step_shape_f16(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats)
 {
-    if (fits32(ns)) step_occupancy_t<__half, float, uint32_t>(scheme, nx, stats, direct, rows);
-    else step_occupancy_t<__half, float, uint64_t>(scheme, nx, stats, direct, rows);
-    if (rows > 0 && rows_fixed<512>(row_plan<__half>(nx), nx)) rows = rows_occupancy_f16_nx512(scheme, stats);
+    StepShape s = fits32(ns) ? step_shape_t<__half, float, uint32_t>(scheme, nx, n, stats)
+                             : step_shape_t<__half, float, uint64_t>(scheme, nx, n, stats);
+    if (s.rows > 0 && rows_fixed<512>(row_plan<__half>(nx), nx)) s.rows = rows_occupancy_f16_nx512(scheme, stats);
+    return s;
 }
 
 }  // namespace flbm

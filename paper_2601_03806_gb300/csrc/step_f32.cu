@@ -18,11 +18,12 @@ cudaError_t launch_step_f32(float *g, const StepArgs<float> &a, int scheme, bool
     return launch_step_t<float, float, uint64_t>(g, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-void step_occupancy_f32(int scheme, uint32_t nx, uint64_t ns, bool stats, int &direct, int &rows)
+StepShape step_shape_f32(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats)
 {
-    if (fits32(ns)) step_occupancy_t<float, float, uint32_t>(scheme, nx, stats, direct, rows);
-    else step_occupancy_t<float, float, uint64_t>(scheme, nx, stats, direct, rows);
-    if (rows > 0 && rows_paced<float>(row_plan<float>(nx))) rows = rows_occupancy_f32_paced(scheme, stats, nx);
+    StepShape s = fits32(ns) ? step_shape_t<float, float, uint32_t>(scheme, nx, n, stats)
+                             : step_shape_t<float, float, uint64_t>(scheme, nx, n, stats);
+    if (s.rows > 0 && rows_paced<float>(row_plan<float>(nx))) s.rows = rows_occupancy_f32_paced(scheme, stats, nx);
+    return s;
 }
 
 }  // namespace flbm

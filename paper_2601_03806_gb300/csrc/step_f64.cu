@@ -10,9 +10,9 @@ cudaError_t launch_step_f64(double *g, const StepArgs<double> &a, int scheme, bo
     return launch_step_t<double, double, uint64_t>(g, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-void step_occupancy_f64(int scheme, uint32_t nx, bool stats, int &direct, int &rows)
+StepShape step_shape_f64(int scheme, uint32_t nx, uint64_t n, uint64_t, bool stats)
 {
-    step_occupancy_t<double, double, uint64_t>(scheme, nx, stats, direct, rows);
+    return step_shape_t<double, double, uint64_t>(scheme, nx, n, stats);
 }
 
 }  // namespace flbm

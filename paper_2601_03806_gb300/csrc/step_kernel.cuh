@@ -43,8 +43,8 @@
 //                barrier sits in the loop.  FP32 / FP16 rows of 256 nodes
 //                and more: a compute thread collides two adjacent nodes at
 //                once (NP = 2); otherwise one (NP = 1).
-//   k_step       (any box): one thread per node, a CTA per 128-node chunk of
-//                a row, direct coalesced loads and stores.
+//   k_step       (any box): nodes in flat order, one or two per thread, direct
+//                coalesced loads and stores.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -375,13 +375,13 @@ __device__ __forceinline__ void normal_pair(uint2 w1, uint2 w2, float2 &rad, flo
 
 // The four normals of Philox block blk as (rad0, c0, s0, rad1, c1, s1):
 // r_{4+4 blk + m} = -(rad0 c0, rad0 s0, rad1 c1, rad1 s1)[m].  V = float2:
-// nodes node and node + 1.
-template <typename V, typename A>
+// nodes node and node + APART.
+template <typename V, int APART = 1, typename A>
 __device__ __forceinline__ void block_normals(const A &a, uint32_t node, int blk, V &rad0, V &c0, V &s0, V &rad1,
                                               V &c1, V &s1)
 {
     if constexpr (std::is_same<V, float2>::value) {
-        const u32x4 oa = noise_block(a, node, blk), ob = noise_block(a, node + 1, blk);
+        const u32x4 oa = noise_block(a, node, blk), ob = noise_block(a, node + APART, blk);
         normal_pair(make_uint2(oa.x, ob.x), make_uint2(oa.y, ob.y), rad0, c0, s0);
         normal_pair(make_uint2(oa.z, ob.z), make_uint2(oa.w, ob.w), rad1, c1, s1);
     } else if constexpr (std::is_same<V, double>::value) {
@@ -551,7 +551,7 @@ __device__ __forceinline__ void collide_modes(V (&v)[3][3][3], const A &a, V (&a
 
 // a6-a7: the node's noise added to the amplitudes qm (destroyed), then the
 // reconstruction into post-collision deviations v (PAIRS as collide_modes).
-template <typename V, bool PREDRAWN, bool PAIRS = true, typename A>
+template <typename V, bool PREDRAWN, bool PAIRS = true, int APART = 1, typename A>
 __device__ __forceinline__ void noise_synthesise(V (&qm)[3][3][3], V rho, const A &a, const V (&nz)[kNoise],
                                                  uint32_t node, V (&v)[3][3][3])
 {
@@ -572,7 +572,7 @@ __device__ __forceinline__ void noise_synthesise(V (&qm)[3][3][3], V rho, const 
 #pragma unroll
             for (int blk = 0; blk < 6; ++blk) {
                 V rad0, c0, s0, rad1, c1, s1;
-                block_normals(a, node, blk, rad0, c0, s0, rad1, c1, s1);
+                block_normals<V, APART>(a, node, blk, rad0, c0, s0, rad1, c1, s1);
                 const V trig[4] = {c0, s0, c1, s1};
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
@@ -621,24 +621,24 @@ __device__ __forceinline__ void noise_synthesise(V (&qm)[3][3][3], V rho, const 
             for (int k = 0; k < 3; ++k) v[i][j][k] = qm[i][j][k];
 }
 
-// a2-a7, a9: collision of one node (V = float2: of nodes node and node + 1,
+// a2-a7, a9: collision of one node (V = float2: of nodes node and node + APART,
 // one per lane).  v[cx+1][cy+1][cz+1] holds the incoming deviations on entry
 // and the post-collision deviations on exit.  PREDRAWN: nz holds the node's
 // scaled normals (draw_noise, drawn before the populations arrived);
 // otherwise the normals of `node` are drawn here pair by pair and folded in
 // at once (fewer live registers).
-template <typename V, int SCHEME, bool STATS, bool PREDRAWN, typename A>
+template <typename V, int SCHEME, bool STATS, bool PREDRAWN, int APART = 1, typename A>
 __device__ __forceinline__ void collide_core(V (&v)[3][3][3], const A &a,
                                              const V (&nz)[kNoise], uint32_t node, V (&acc)[NSTAT])
 {
     V qm[3][3][3];
     V rho, dj[4];
     collide_modes<V, SCHEME, STATS, !std::is_same<V, float2>::value>(v, a, acc, qm, rho, dj);
-    noise_synthesise<V, PREDRAWN, !std::is_same<V, float2>::value>(qm, rho, a, nz, node, v);
+    noise_synthesise<V, PREDRAWN, !std::is_same<V, float2>::value, APART>(qm, rho, a, nz, node, v);
 }
 
 // ---------------------------------------------------------------------------
-// k_step: one thread per node, direct loads/stores (general boxes)
+// k_step: direct loads/stores (general boxes)
 
 // Periodic neighbour offsets of node (x,y,z): xs[d], ry[d], rz[d] for the
 // displacements d-1 = -1, 0, +1 along each axis (node index = xs + ry + rz).
@@ -662,58 +662,186 @@ struct Nbr {
     __device__ __forceinline__ I node() const { return xs[1] + ry[1] + rz[1]; }
 };
 
-template <typename S, typename R, typename I, int SCHEME, bool ODD, bool STATS>
-__global__ void __launch_bounds__(kBlock, FLBM_MIN_BLOCKS) k_step(S *__restrict__ g, const StepArgs<R> a)
+// A position (x, y, z) stepped by a fixed number of nodes in flat order,
+// itself as (x, y, z) in the same mixed radix: two carries, no division.
+struct NodeWalk {
+    uint32_t x, y, z;
+    template <typename R>
+    __device__ __forceinline__ NodeWalk(const StepArgs<R> &a, uint64_t n)
+    {
+        if (n <= 0xffffffffull) {   // 32-bit divisions
+            const uint32_t m = uint32_t(n), r = m / a.nx;
+            x = m - r * a.nx;
+            z = r / a.ny;
+            y = r - z * a.ny;
+            return;
+        }
+        const uint64_t r = n / a.nx;
+        x = uint32_t(n % a.nx);
+        y = uint32_t(r % a.ny);
+        z = uint32_t(r / a.ny);
+    }
+    template <typename R>
+    __device__ __forceinline__ void next(const StepArgs<R> &a, const NodeWalk &d)
+    {
+        x += d.x;
+        y += d.y;
+        z += d.z;
+        if (x >= a.nx) {
+            x -= a.nx;
+            ++y;
+        }
+        if (y >= a.ny) {
+            y -= a.ny;
+            ++z;
+        }
+    }
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+// 4-byte copies from global to shared memory, in groups of the thread's own.
+__device__ __forceinline__ void cp_async4(float *dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Element index of population c = (i - 1, j - 1, k - 1) of node n, with
+// neighbours nb, as the AA pattern reads it (LOAD) or writes it.
+template <typename I, bool ODD, bool LOAD>
+__device__ __forceinline__ I pop_index(const Nbr<I> &nb, I n, I N, int i, int j, int k)
+{
+    if (ODD != LOAD) {   // slot of c
+        const I slab = I(slot_of(i - 1, j - 1, k - 1)) * N;
+        return slab + (ODD ? nb.xs[i] + nb.ry[j] + nb.rz[k] : n);
+    }
+    const I slab = I(slot_of(1 - i, 1 - j, 1 - k)) * N;
+    return slab + (ODD ? nb.xs[2 - i] + nb.ry[2 - j] + nb.rz[2 - k] : n);
+}
+
+// The direct kernel: nodes are taken in flat order, so rows of any length
+// fill the warps (a CTA per 128-node piece of a row left 7 of 8 threads of a
+// 16-node row idle).  NP = 1: thread t of a CTA takes node base + t.  NP = 2
+// (FP32 arithmetic): nodes base + t and base + t + 128, one per lane of packed
+// FP32 pairs, which keeps both accesses coalesced and aligned whatever the
+// row length.  FP32 storage at NP = 2 is staged: while a thread collides its
+// two nodes, 4-byte cp.async bring the next two into its own column of shared
+// memory (no barrier: no other thread touches it; and reading early is safe
+// in place, a node's AA reads are exactly its own writes), so the loads of 54
+// populations wait behind the collision instead of in front of it.
+// What bounds it: instruction issue (800-915 a node, a quarter more than the
+// row kernels, for the 108 accesses of two nodes) with 12 warps per SM; DRAM
+// at 57-64 % of its peak.  250 x 243 x 121 FP32: 326 us a step (22.5 GLUPS),
+// 374 with one node per thread in row chunks; 100^3 51 us instead of 76; 16^3
+// 8 instead of 21.  Unstaged: 332 us, and 56 us at 100^3.
+template <typename S, typename R, typename I, int SCHEME, bool ODD, bool STATS, int NP>
+__global__ void __launch_bounds__(kBlock, NP == 2 ? 3 : FLBM_MIN_BLOCKS) k_step(S *__restrict__ g, const StepArgs<R> a)
+{
+    using V = typename std::conditional<NP == 2, float2, R>::type;
+    constexpr bool STAGED = NP == 2 && sizeof(S) == 4;
     __shared__ TotSlot<R> tot[32][NSTAT];
-    R acc[NSTAT];
+    __shared__ float2 column[STAGED ? kQ : 1][kBlock];
+    V acc[NSTAT];
 #pragma unroll
-    for (int s = 0; s < NSTAT; ++s) acc[s] = R(0);
+    for (int s = 0; s < NSTAT; ++s) acc[s] = vset<V>(0.0);
     if (STATS) {
         totals_init(tot);
         __syncthreads();
     }
     const I N = I(a.ns);   // slab stride
+    // NP = 2 runs whole CTAs of kBlock threads, NP = 1 CTAs of any size
+    const uint32_t threads = NP == 2 ? uint32_t(kBlock) : blockDim.x;
+    const uint64_t stride = uint64_t(gridDim.x) * (threads * NP);
+    uint64_t n = uint64_t(blockIdx.x) * (threads * NP) + threadIdx.x;   // lane .x's node
+    NodeWalk wa(a, n), wb(a, NP == 2 ? n + kBlock : n);
+    const NodeWalk step(a, stride);
+    // f(i, j, k, element of lane .x, of lane .y) for the populations of the
+    // nodes m (at wa) and m + kBlock (at wb; only meaningful if it exists)
+    auto each = [&](auto load, uint64_t m, bool two, auto &&f) {
+        constexpr bool LOAD = decltype(load)::value;
+        const Nbr<I> nb(wa.x, wa.y, wa.z, a.nx, a.ny, a.nz);
+        const Nbr<I> nb2(two ? wb.x : 0, two ? wb.y : 0, two ? wb.z : 0, a.nx, a.ny, a.nz);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    f(i, j, k, pop_index<I, ODD, LOAD>(nb, I(m), N, i, j, k),
+                      NP == 2 ? pop_index<I, ODD, LOAD>(nb2, I(m) + kBlock, N, i, j, k) : I(0));
+    };
+    auto stage = [&](uint64_t m) {
+        if constexpr (STAGED) {
+            if (m < a.n) {
+                const bool two = m + kBlock < a.n;
+                each(std::true_type{}, m, two, [&](int i, int j, int k, I e, I e2) {
+                    float2 *c = &column[9 * i + 3 * j + k][threadIdx.x];
+                    cp_async4(&c->x, reinterpret_cast<const float *>(g) + e);
+                    if (two) cp_async4(&c->y, reinterpret_cast<const float *>(g) + e2);
+                    else c->y = 0.0f;
+                });
+            }
+            cp_async_commit();
+        }
+    };
+    stage(n);
     uint32_t it = 0;
-    for (uint64_t ch = blockIdx.x; ch < a.nchunks; ch += gridDim.x, ++it) {
-        // CTA-uniform: every thread walks the same chunks
+    for (uint64_t base = n - threadIdx.x; base < a.n; base += stride, n += stride, ++it) {
+        // CTA-uniform: every thread walks the same groups
         if (STATS && it % kFlushEvery == kFlushEvery - 1) warp_flush(acc, tot);
-        const uint32_t xc = uint32_t(ch % a.cpr);
-        const uint64_t r = ch / a.cpr;
-        const uint32_t y = uint32_t(r % a.ny);
-        const uint32_t z = uint32_t(r / a.ny);
-        const uint32_t x = xc * kBlock + threadIdx.x;
-        if (x >= a.nx) continue;
-        const Nbr<I> nb(x, y, z, a.nx, a.ny, a.nz);
-        const I n = nb.node();
+        // a node past the end reads zeros (which add nothing to the sums) and
+        // stores nothing
+        const bool on = n < a.n, on2 = NP == 2 && n + kBlock < a.n;
+        V v[3][3][3];
         // a1: load
-        R v[3][3][3];
+        if constexpr (STAGED) {
+            cp_async_wait_all();
+            if (on) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
+                    for (int j = 0; j < 3; ++j)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    I idx;
-                    if (!ODD) idx = I(slot_of(i - 1, j - 1, k - 1)) * N + n;
-                    else idx = I(slot_of(1 - i, 1 - j, 1 - k)) * N + (nb.xs[2 - i] + nb.ry[2 - j] + nb.rz[2 - k]);
-                    v[i][j][k] = Conv<S, R>::ld(g + idx);
+                        for (int k = 0; k < 3; ++k) v[i][j][k] = column[9 * i + 3 * j + k][threadIdx.x];
+            }
+        } else if (on) {
+            each(std::true_type{}, n, on2, [&](int i, int j, int k, I e, I e2) {
+                if constexpr (NP == 2) {
+                    v[i][j][k].x = Conv<S, R>::ld(g + e);
+                    v[i][j][k].y = on2 ? Conv<S, R>::ld(g + e2) : 0.0f;
+                } else {
+                    v[i][j][k] = Conv<S, R>::ld(g + e);
                 }
-        R nz[kNoise];   // unused: the direct kernel draws the normals inside
-        collide_core<R, SCHEME, STATS, false>(v, a, nz, uint32_t(n), acc);
-        // a8: AA store
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    I idx;
-                    if (!ODD) idx = I(slot_of(1 - i, 1 - j, 1 - k)) * N + n;
-                    else idx = I(slot_of(i - 1, j - 1, k - 1)) * N + (nb.xs[i] + nb.ry[j] + nb.rz[k]);
-                    Conv<S, R>::st(g + idx, v[i][j][k]);
+            });
+        }
+        const NodeWalk ca = wa, cb = wb;
+        wa.next(a, step);
+        if (NP == 2) wb.next(a, step);
+        stage(n + stride);
+        if (on) {
+            V nz[kNoise];   // unused: the direct kernel draws the normals inside
+            collide_core<V, SCHEME, STATS, false, kBlock>(v, a, nz, uint32_t(n), acc);
+            // a8: AA store
+            const NodeWalk na = wa, nb = wb;
+            wa = ca;
+            wb = cb;
+            each(std::false_type{}, n, on2, [&](int i, int j, int k, I e, I e2) {
+                if constexpr (NP == 2) {
+                    Conv<S, R>::st(g + e, v[i][j][k].x);
+                    if (on2) Conv<S, R>::st(g + e2, v[i][j][k].y);
+                } else {
+                    Conv<S, R>::st(g + e, v[i][j][k]);
                 }
+            });
+            wa = na;
+            wb = nb;
+        }
     }
+    if (STAGED) cp_async_wait_all();   // no copy may land after the CTA has left
     if (STATS) {
         warp_flush(acc, tot);
         block_store_totals(tot, a.partials + size_t(blockIdx.x) * NSTAT);
@@ -723,10 +851,6 @@ __global__ void __launch_bounds__(kBlock, FLBM_MIN_BLOCKS) k_step(S *__restrict_
 // ---------------------------------------------------------------------------
 // k_step_rows: TMA bulk-copy row pipeline
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count));
@@ -1148,6 +1272,36 @@ void launch_rows(S *g, const StepArgs<R> &a, const RowPlan &rp, int row_grid, cu
     k_step_rows<S, R, SC, OD, ST, 1><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2);
 }
 
+template <typename S, typename R, typename I, int SC, bool OD, bool ST, typename Plan>
+void launch_direct(S *g, const StepArgs<R> &a, const Plan &dp, int grid, cudaStream_t s)
+{
+    if constexpr (!std::is_same<S, double>::value) {
+        if (dp.np == 2) {
+            k_step<S, R, I, SC, OD, ST, 2><<<grid, dp.threads, 0, s>>>(g, a);
+            return;
+        }
+    }
+    k_step<S, R, I, SC, OD, ST, 1><<<grid, dp.threads, 0, s>>>(g, a);
+}
+
+// Shape of the direct kernel for a box of n nodes: nodes and threads per CTA.
+// Boxes that leave the chip idle are spread over more, smaller CTAs of one
+// node a thread.
+struct DirectPlan {
+    int np, threads;
+    uint64_t ctas;
+};
+template <typename S>
+inline DirectPlan direct_plan(uint64_t n)
+{
+    DirectPlan p;
+    p.np = !std::is_same<S, double>::value && row_pairs_enabled() && n >= kDirectPairs ? 2 : 1;
+    p.threads = n >= kDirectPairs ? kBlock : 32;
+    const uint64_t span = uint64_t(p.np) * p.threads;
+    p.ctas = (n + span - 1) / span;
+    return p;
+}
+
 template <typename S, typename R, typename I>
 cudaError_t launch_step_t(S *g, const StepArgs<R> &a, int scheme, bool odd, bool stats, int grid,
                           int row_grid, cudaStream_t s)
@@ -1168,7 +1322,8 @@ cudaError_t launch_step_t(S *g, const StepArgs<R> &a, int scheme, bool odd, bool
 #undef FLBM_LAUNCH_ROWS
         return cudaGetLastError();
     }
-#define FLBM_LAUNCH(SC, OD, ST) k_step<S, R, I, SC, OD, ST><<<grid, kBlock, 0, s>>>(g, a)
+    const DirectPlan dp = direct_plan<S>(a.n);
+#define FLBM_LAUNCH(SC, OD, ST) launch_direct<S, R, I, SC, OD, ST>(g, a, dp, grid, s)
     if (scheme == 0) {
         if (odd) { if (stats) FLBM_LAUNCH(0, true, true); else FLBM_LAUNCH(0, true, false); }
         else     { if (stats) FLBM_LAUNCH(0, false, true); else FLBM_LAUNCH(0, false, false); }
@@ -1251,38 +1406,51 @@ int prepare_rows_fixed(int scheme, bool stats, uint32_t nx = NXC)
     return prepare_rows<S, R, 2, 2, NXC, PACED>(rp, stats);
 }
 
-// Resident CTAs per SM of the larger (reducing, odd-form) variant of each
-// kernel; also opts the row kernels into their shared memory on the current
-// device.  rows = 0 when the row pipeline does not serve the box.
-template <typename S, typename R, typename I, int SC>
-void prepare_scheme(uint32_t nx, bool stats, int &direct, int &rows)
+// CTAs of the direct kernel that an SM keeps resident (of the larger, odd-form
+// variant) for plan dp.
+template <typename S, typename R, typename I, int SC, int NP>
+int direct_resident(const DirectPlan &dp, bool stats)
 {
-    direct = 1;
-    rows = 0;
     int nb = 0;
-    cudaError_t e = stats
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<S, R, I, SC, true, true>, kBlock, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<S, R, I, SC, true, false>, kBlock, 0);
-    if (e == cudaSuccess && nb > 0) direct = nb;
+    const cudaError_t e = stats
+        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<S, R, I, SC, true, true, NP>, dp.threads, 0)
+        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<S, R, I, SC, true, false, NP>, dp.threads, 0);
+    return e == cudaSuccess && nb > 0 ? nb : 1;
+}
+
+// The step kernels of a box of n nodes in rows of nx: the direct kernel's
+// CTAs in all and resident per SM, and the row kernel's per SM (0 when the
+// row pipeline does not serve the box); also opts the row kernels into their
+// shared memory on the current device.
+template <typename S, typename R, typename I, int SC>
+void prepare_scheme(uint32_t nx, uint64_t n, bool stats, StepShape &shape)
+{
+    const DirectPlan dp = direct_plan<S>(n);
+    shape.ctas = dp.ctas;
+    shape.rows = 0;
+    if constexpr (std::is_same<S, double>::value) shape.direct = direct_resident<S, R, I, SC, 1>(dp, stats);
+    else shape.direct = dp.np == 2 ? direct_resident<S, R, I, SC, 2>(dp, stats) : direct_resident<S, R, I, SC, 1>(dp, stats);
     const RowPlan rp = row_plan<S>(nx);
     if (!rp.use) return;
     // the attribute is per kernel, shared by every context of the process:
     // set it to the largest staging any box may use, not to this box's
     if constexpr (!std::is_same<S, double>::value) {
         if (rp.np == 2) {
-            rows = prepare_rows<S, R, SC, 2>(rp, stats);
+            shape.rows = prepare_rows<S, R, SC, 2>(rp, stats);
             return;
         }
     }
-    rows = prepare_rows<S, R, SC, 1>(rp, stats);
+    shape.rows = prepare_rows<S, R, SC, 1>(rp, stats);
 }
 
 template <typename S, typename R, typename I>
-void step_occupancy_t(int scheme, uint32_t nx, bool stats, int &direct, int &rows)
+StepShape step_shape_t(int scheme, uint32_t nx, uint64_t n, bool stats)
 {
-    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, stats, direct, rows);
-    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, stats, direct, rows);
-    else prepare_scheme<S, R, I, 2>(nx, stats, direct, rows);
+    StepShape shape;
+    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, n, stats, shape);
+    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, n, stats, shape);
+    else prepare_scheme<S, R, I, 2>(nx, n, stats, shape);
+    return shape;
 }
 
 }  // namespace flbm

@@ -75,13 +75,6 @@ __device__ __forceinline__ Site site_of(const Walk &w, const StepArgs<float> &a)
     return s;
 }
 
-__device__ __forceinline__ void cp_async4(float *dst, const float *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
 // Population c = (i-1, j-1, k-1) of node (x, y, z) as the AA pattern reads it.
 template <typename I, bool ODD>
 __device__ __forceinline__ I load_index(const Nbr<I> &nb, I N, int i, int j, int k)
