@@ -397,7 +397,7 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
     const auto step_shape = p->precision == FLBM_FP64   ? step_shape_f64
                             : p->precision == FLBM_FP32 ? step_shape_f32
                                                         : step_shape_f16;
-    step_grids(*p, c->nsm, step_shape(p->scheme, uint32_t(p->nx), c->n, c->ns, true), c->grid, c->row_grid);
+    step_grids(*p, c->nsm, step_shape(p->scheme, uint32_t(p->nx), uint32_t(p->ny), uint32_t(p->nz), c->ns, true), c->grid, c->row_grid);
     // FLBM_INJECT_STARVE=1 (environment, failure-injection tests only): the
     // row pipeline expects 16 bytes more than it copies (the learned step
     // issues no first-layer MMA), so the bounded waits run out and flbm_step
@@ -457,12 +457,14 @@ void step_grids(const flbm_params &p, int nsm, const StepShape &shape, int &grid
     if (p.scheme == FLBM_LEARNED) per_sm = learned_occupancy(n);
     grid = int(std::min<uint64_t>(work, uint64_t(nsm) * per_sm));
     if (grid < 1) grid = 1;
-    // FLBM_ROWS=0 (environment) disables the TMA row pipeline
+    // FLBM_ROWS (environment): 0 disables the TMA row pipeline, 1 runs it for
+    // small boxes too, as failure injection does (its waits are what runs out)
     row_grid = 0;
-    const char *rows_env = std::getenv("FLBM_ROWS");
-    if (shape.rows > 0 && p.scheme != FLBM_LEARNED && !(rows_env && std::atoi(rows_env) == 0)) {
-        const uint64_t nrows = uint64_t(p.ny) * p.nz;
-        row_grid = int(std::min<uint64_t>(nrows, uint64_t(nsm) * shape.rows));
+    const char *rows_env = std::getenv("FLBM_ROWS"), *inject = std::getenv("FLBM_INJECT_STARVE");
+    const int rows = rows_env ? std::atoi(rows_env) : (inject && std::atoi(inject) == 1 ? 1 : -1);
+    const bool small = n < (p.precision == FLBM_FP64 ? kRowsFrom64 : kRowsFrom);
+    if (shape.rows > 0 && p.scheme != FLBM_LEARNED && rows != 0 && (rows == 1 || !small)) {
+        row_grid = int(std::min<uint64_t>(shape.work, uint64_t(nsm) * shape.rows));
     }
 }
 

@@ -154,30 +154,40 @@ cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool 
 // Nodes from which the direct kernel takes two per thread in CTAs of kBlock
 // threads (below, one per thread in CTAs of a warp).
 constexpr uint64_t kDirectPairs = 65536;
-// Launch shape of the step kernels for a box of n nodes in rows of nx: the
-// direct kernel's CTAs and how many of them an SM holds, and the row
+// Launch shape of the step kernels for a box: the direct kernel's CTAs and how many of them an SM holds, and the row
 // pipeline's CTAs per SM (0 when it does not serve rows of length nx); the
 // slab stride ns picks the index width.  Also prepares the kernels'
 // shared-memory attributes on the current device.
 struct StepShape {
-    uint64_t ctas = 1;
+    uint64_t ctas = 1, work = 0;   // of the direct kernel; work items of the row pipeline
     int direct = 1, rows = 0;
 };
-StepShape step_shape_f64(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
-StepShape step_shape_f32(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
-StepShape step_shape_f16(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats);
+StepShape step_shape_f64(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
+StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
+StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
+// Nodes from which boxes whose rows the pipeline can take run it (FP32 / FP16,
+// FP64); smaller ones run the direct kernel, which needs no fill and drain.
+constexpr uint64_t kRowsFrom = uint64_t(1) << 19, kRowsFrom64 = uint64_t(1) << 16;
+// The grouped-row kernels (step_f32_items.cu, step_f16_items.cu) of boxes
+// whose row_plan is grouped.
+cudaError_t launch_items_f32(float *g, const StepArgs<float> &a, int scheme, bool odd, bool stats, int row_grid,
+                             cudaStream_t s);
+cudaError_t launch_items_f16(void *g, const StepArgs<float> &a, int scheme, bool odd, bool stats, int row_grid,
+                             cudaStream_t s);
+int items_resident_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz);
+int items_resident_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz);
 // The FP16-storage two-node row kernels for rows of exactly 512 nodes
 // (step_f16_nx512.cu), which step_f16.cu calls when the row plan of the box
 // takes two nodes per thread in full CTAs.  FP32 keeps the general kernel:
 // there the step is at the HBM bound and the fixed length gains nothing.
 cudaError_t launch_rows_f16_nx512(void *g, const StepArgs<float> &a, int scheme, bool odd, bool stats,
                                   int row_grid, cudaStream_t s);
-int rows_occupancy_f16_nx512(int scheme, bool stats);
+int rows_occupancy_f16_nx512(int scheme, bool stats, uint32_t ny, uint32_t nz);
 // The PACED FP32 two-node row kernels (step_f32_paced.cu) for rows staged
 // twice, which step_f32.cu calls when rows_paced<float> holds for the box.
 cudaError_t launch_rows_f32_paced(float *g, const StepArgs<float> &a, int scheme, bool odd, bool stats,
                                   int row_grid, cudaStream_t s);
-int rows_occupancy_f32_paced(int scheme, bool stats, uint32_t nx);
+int rows_occupancy_f32_paced(int scheme, bool stats, uint32_t nx, uint32_t ny, uint32_t nz);
 
 // Step constants shared by flbm_step and flbm_step_noalloc (capi.cu): the
 // Philox round keys, the density used by the noise, and the per-mode

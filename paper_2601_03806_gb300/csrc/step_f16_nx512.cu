@@ -14,9 +14,9 @@ cudaError_t launch_rows_f16_nx512(void *g, const StepArgs<float> &a, int scheme,
     return launch_rows_fixed<__half, float, 512>(static_cast<__half *>(g), a, scheme, odd, stats, row_grid, s);
 }
 
-int rows_occupancy_f16_nx512(int scheme, bool stats)
+int rows_occupancy_f16_nx512(int scheme, bool stats, uint32_t ny, uint32_t nz)
 {
-    return prepare_rows_fixed<__half, float, 512>(scheme, stats);
+    return prepare_rows_fixed<__half, float, 512>(scheme, stats, row_plan<__half>(512, ny, nz));
 }
 
 }  // namespace flbm

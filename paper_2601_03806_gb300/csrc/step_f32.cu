@@ -11,18 +11,27 @@ static bool fits32(uint64_t n) { return n * kQ < (1ull << 32); }
 cudaError_t launch_step_f32(float *g, const StepArgs<float> &a, int scheme, bool odd, bool stats,
                             int grid, int row_grid, cudaStream_t s)
 {
-    if (row_grid > 0 && rows_paced<float>(row_plan<float>(a.nx)))
-        return launch_rows_f32_paced(g, a, scheme, odd, stats, row_grid, s);
+    if (row_grid > 0) {
+        const RowPlan rp = row_plan<float>(a.nx, a.ny, a.nz);
+        if (rp.grouped) return launch_items_f32(g, a, scheme, odd, stats, row_grid, s);
+        if (rows_paced<float>(rp)) return launch_rows_f32_paced(g, a, scheme, odd, stats, row_grid, s);
+    }
     if (fits32(a.ns))
         return launch_step_t<float, float, uint32_t>(g, a, scheme, odd, stats, grid, row_grid, s);
     return launch_step_t<float, float, uint64_t>(g, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-StepShape step_shape_f32(int scheme, uint32_t nx, uint64_t n, uint64_t ns, bool stats)
+StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats)
 {
-    StepShape s = fits32(ns) ? step_shape_t<float, float, uint32_t>(scheme, nx, n, stats)
-                             : step_shape_t<float, float, uint64_t>(scheme, nx, n, stats);
-    if (s.rows > 0 && rows_paced<float>(row_plan<float>(nx))) s.rows = rows_occupancy_f32_paced(scheme, stats, nx);
+    StepShape s = fits32(ns) ? step_shape_t<float, float, uint32_t>(scheme, nx, ny, nz, stats)
+                             : step_shape_t<float, float, uint64_t>(scheme, nx, ny, nz, stats);
+    const RowPlan rp = row_plan<float>(nx, ny, nz);
+    if (rp.grouped) {
+        s.rows = items_resident_f32(scheme, nx, ny, nz);
+        s.work = rp.work;
+    } else if (rows_paced<float>(rp)) {
+        s.rows = rows_occupancy_f32_paced(scheme, stats, nx, ny, nz);
+    }
     return s;
 }
 

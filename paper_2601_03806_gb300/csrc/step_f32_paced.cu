@@ -12,9 +12,9 @@ cudaError_t launch_rows_f32_paced(float *g, const StepArgs<float> &a, int scheme
     return launch_rows_fixed<float, float, 0, true>(g, a, scheme, odd, stats, row_grid, s);
 }
 
-int rows_occupancy_f32_paced(int scheme, bool stats, uint32_t nx)
+int rows_occupancy_f32_paced(int scheme, bool stats, uint32_t nx, uint32_t ny, uint32_t nz)
 {
-    return prepare_rows_fixed<float, float, 0, true>(scheme, stats, nx);
+    return prepare_rows_fixed<float, float, 0, true>(scheme, stats, row_plan<float>(nx, ny, nz));
 }
 
 }  // namespace flbm

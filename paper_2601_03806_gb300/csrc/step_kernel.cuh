@@ -27,7 +27,7 @@
 //   a9  optional per-thread partial sums of the reductions, folded per warp
 //       every 8 rows into exact (hi, lo) slots and summed per CTA in FP64
 //
-// Two kernels move the data (a1 load, a8 store):
+// Three kernels move the data (a1 load, a8 store):
 //   k_step_rows  (rows whose x-extent is a multiple of 32 and fits shared
 //                memory): a persistent, warp-specialised CTA owns whole
 //                x-rows.  Its producer warp moves, per row, the 27 aligned
@@ -40,15 +40,18 @@
 //                its write set) and release the stage on an "empty"
 //                mbarrier; the producer then bulk-stores the segments back.
 //                All HBM traffic is aligned bulk transfers and no CTA-wide
-//                barrier sits in the loop.  FP32 / FP16 rows of 256 nodes
-//                and more: a compute thread collides two adjacent nodes at
-//                once (NP = 2); otherwise one (NP = 1).
+//                barrier sits in the loop.  FP32 / FP16 rows of more than 256
+//                nodes: a compute thread collides two adjacent nodes at once
+//                (NP = 2); FP64 and longer rows: one (NP = 1).
+//   k_step_items (FP32 / FP16 rows of 32 to 256 nodes): the same pipeline with
+//                several rows to a work item, two nodes per thread.
 //   k_step       (any box): nodes in flat order, one or two per thread, direct
 //                coalesced loads and stores.
 #pragma once
 
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.h"
@@ -1026,10 +1029,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // shared-memory access instead of an address computed per access.
 // PACED: the copy warp derives every copy's address from the row index
 // (row_segment_paced) instead of walking the rows (RowWalk): the same
-// addresses, issued more slowly.  Launched for the FP32 two-node rows
-// staged twice (288-512 nodes; the HBM-bound 512^3 step), where walking made
-// the step 1.5-2.1 % slower; everywhere else walking is faster (256^3 FP32
-// +10.8 %, 128^3 FP32 +8.3 %, 512^3 FP16 +2.5 %).
+// addresses, issued more slowly.  Launched for the FP32 two-node rows (288-512 nodes; the HBM-bound 512^3 step), where walking made the step
+// 1.5-2.1 % slower; in the other kernels walking is faster (512^3 FP16 +2.5
+// %).
 template <typename S, typename R, int SCHEME, bool ODD, bool STATS, int NP, uint32_t NXC = 0, bool PACED = false>
 __global__ void __launch_bounds__(NP == 2 ? kRowPairCompute + 32 : kRowCompute + 32,
                                   NP == 2 ? row_pair_ctas<S>() : (sizeof(S) <= 4 ? 2 : 1))
@@ -1217,32 +1219,210 @@ __global__ void __launch_bounds__(NP == 2 ? kRowPairCompute + 32 : kRowCompute +
 }
 
 // ---------------------------------------------------------------------------
+// k_step_items: the two-node row pipeline for rows of up to 256 nodes.  A work
+// item is `rows` consecutive x-rows of one z-plane (fewer at the plane's end),
+// kItemNodes nodes at most, staged as 27 segments of kItemNodes elements (a
+// compile-time stride: the segment offsets are immediates).  Rows follow one
+// another in memory, so a segment is one bulk copy, or two where the odd
+// form's rows y - cy wrap around the plane.  What bounds it: HBM for large
+// boxes (128 x 512 x 512 FP32 96 % of the copy rate), the last round of items
+// for small ones.  512 nodes in two stages, because an item's waits and
+// barriers cost the same whatever its size: 128^3 FP32 83 us a step, 90 us
+// with four stages of 256, 96 us with a row per item and a node per thread
+// (128 x 256 x 256: 289, 330 and 356 us; 32 x 512 x 512: 291, 333 and 589).
+constexpr uint32_t kItemNodes = 512;
+
+struct RowItems {
+    uint32_t rows, per_plane;   // rows of an item, items of a plane
+};
+
+template <typename S, typename R, int SCHEME, bool ODD, bool STATS>
+__global__ void __launch_bounds__(kRowPairCompute + 32, row_pair_ctas<S>())
+    k_step_items(S *__restrict__ g, const StepArgs<R> a, const RowItems items)
+{
+    constexpr uint32_t nc = kRowPairCompute, stage_elems = uint32_t(kQ) * kItemNodes;
+    // a thread's nodes between two flushes: those of kFlushEvery 256-node rows
+    constexpr uint32_t kFlush = kFlushEvery * 256 / kItemNodes;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full[2], empty[2];
+    __shared__ TotSlot<R> tot[32][NSTAT];
+    constexpr uint32_t nst = 2;   // stages
+    S *const stage = reinterpret_cast<S *>(smem_raw);
+    const uint32_t lane = threadIdx.x & 31, nx = a.nx;
+    float2 acc[NSTAT];
+#pragma unroll
+    for (int s = 0; s < NSTAT; ++s) acc[s] = vset<float2>(0.0);
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < nst; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], nc / 32);
+        }
+        mbar_init_fence();
+    }
+    if (STATS) totals_init(tot);
+    __syncthreads();
+    auto rows_of = [&](uint32_t y0) { return min(items.rows, a.ny - y0); };
+
+    if (threadIdx.x >= nc) {
+        // ---------------- copy warp: lane d moves segment d ----------------
+        const int d = int(lane);
+        const SegLane L = seg_lane<R, ODD>(a, d < kQ ? d : 0);
+        RowWalk wl(items.per_plane), ws(items.per_plane);   // the items loaded / stored next
+        uint64_t k = 0;
+        bool ok = true;
+        auto move = [&](const RowWalk &w, uint32_t s, bool load) {
+            const uint32_t y0 = w.y * items.rows, rows = rows_of(y0);
+            // the first row in memory, and how many follow before the seam
+            uint32_t yy = y0, zz = w.z;
+            if (L.cy > 0) yy = y0 ? y0 - 1 : a.ny - 1;
+            if (L.cy < 0) yy = (y0 + 1 < a.ny) ? y0 + 1 : 0;
+            if (L.cz > 0) zz = w.z ? w.z - 1 : a.nz - 1;
+            if (L.cz < 0) zz = (w.z + 1 < a.nz) ? w.z + 1 : 0;
+            const uint32_t first = min(rows, a.ny - yy);
+            S *const plane = g + (L.slot_off + uint64_t(zz) * a.ny * nx);
+            S *const sp = stage + size_t(s) * stage_elems + uint32_t(d) * kItemNodes;
+            const uint32_t b0 = first * nx * uint32_t(sizeof(S)), b1 = (rows - first) * nx * uint32_t(sizeof(S));
+            if (load) {
+                bulk_g2s(sp, plane + uint64_t(yy) * nx, b0, &full[s]);
+                if (b1) bulk_g2s(sp + first * nx, plane, b1, &full[s]);
+            } else {
+                bulk_s2g(plane + uint64_t(yy) * nx, sp, b0);
+                if (b1) bulk_s2g(plane, sp + first * nx, b1);
+            }
+        };
+        // item number kk of this CTA out of its stage; called for kk = 0, 1, ...
+        auto store_item = [&](uint64_t kk) {
+            const uint32_t s = uint32_t(kk) & (nst - 1);
+            ok = mbar_wait(&empty[s], uint32_t((kk / nst) & 1));
+            if (!ok) return;
+            if (d < kQ) {
+                move(ws, s, false);
+                bulk_commit();
+                bulk_wait_read_all();
+            }
+            ws.next(items.per_plane);
+            __syncwarp();
+        };
+        for (;; ++k, wl.next(items.per_plane)) {
+            if (wl.z >= a.nz) break;
+            const uint32_t s = uint32_t(k) & (nst - 1);
+            if (k >= nst) {
+                store_item(k - nst);
+                if (!ok) break;
+            }
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                mbar_arrive_expect_tx(&full[s], uint32_t(kQ) * rows_of(wl.y * items.rows) * nx * uint32_t(sizeof(S)) +
+                                                    a.tx_pad);
+            }
+            __syncwarp();
+            if (d < kQ) move(wl, s, true);
+        }
+        // drain the last stages
+        for (uint64_t kk = (k > nst ? k - nst : 0); ok && kk < k; ++kk) store_item(kk);
+        if (!ok && lane == 0) atomicOr(a.flag, 2u);
+        if (d < kQ) bulk_wait_all();
+    } else {
+        // ---------------- compute warps, two adjacent nodes of a row per thread ----------------
+        // row of local node l: (l + 1/2) / nx in FP32 is within 512 x 2^-23 of
+        // its exact value and at least 1/(2 nx) from an integer (nx < 512), so
+        // truncation gives l / nx exactly
+        const float inv_nx = __frcp_rn(float(nx));
+        RowWalk w(items.per_plane);
+        for (uint64_t k = 0;; ++k, w.next(items.per_plane)) {
+            if (w.z >= a.nz) break;
+            const uint32_t s = uint32_t(k) & (nst - 1), y0 = w.y * items.rows;
+            const uint32_t base = nx * (y0 + a.ny * w.z), count = rows_of(y0) * nx;
+            // the outcome is made warp-uniform: warp_flush needs every lane
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], uint32_t((k / nst) & 1)))) {
+                if (lane == 0) atomicOr(a.flag, 2u);
+                break;
+            }
+            S *const st = stage + size_t(s) * stage_elems;
+#pragma unroll 1
+            for (uint32_t l = 2 * threadIdx.x; l < count; l += 2 * nc) {
+                // nodes l (lane .x) and l + 1 (lane .y) of one row: l and nx are even
+                const uint32_t t = uint32_t((float(l) + 0.5f) * inv_nx), rb = t * nx, x = l - rb;
+                const uint32_t xa[3] = {rb + (x ? x - 1 : nx - 1), l, l + 1};
+                const uint32_t xb[3] = {l, l + 1, rb + ((x + 2 < nx) ? x + 2 : 0)};
+                float2 v[3][3][3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+#pragma unroll
+                        for (int kk = 0; kk < 3; ++kk) {
+                            const S *seg = st + (9 * i + 3 * j + kk) * kItemNodes;
+                            if (!ODD || i == 1) v[i][j][kk] = ld_pair(seg + l);
+                            else v[i][j][kk] = make_float2(stage_ld(seg[xa[2 - i]]), stage_ld(seg[xb[2 - i]]));
+                        }
+                float2 nz[kNoise];   // unused: the normals are drawn inside, pair by pair
+                collide_core<float2, SCHEME, STATS, false>(v, a, nz, base + l, acc);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+#pragma unroll
+                        for (int kk = 0; kk < 3; ++kk) {
+                            S *seg = st + (9 * (2 - i) + 3 * (2 - j) + (2 - kk)) * kItemNodes;
+                            if (!ODD || i == 1) st_pair(seg + l, v[i][j][kk]);
+                            else {
+                                seg[xa[i]] = stage_st<S>(v[i][j][kk].x);
+                                seg[xb[i]] = stage_st<S>(v[i][j][kk].y);
+                            }
+                        }
+            }
+            fence_proxy_async_smem();   // generic-proxy writes before the bulk store reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[s]);
+            if (STATS && k % kFlush == kFlush - 1) warp_flush(acc, tot);
+        }
+    }
+    if (STATS) {
+        warp_flush(acc, tot);
+        block_store_totals(tot, a.partials + size_t(blockIdx.x) * NSTAT);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // launchers
 
 // Dynamic shared memory of a row-pipeline CTA at most.
 constexpr size_t kRowMaxSmem = 200 * 1024;
 
-// Whether the row pipeline serves a box of row length nx, and its CTA shape:
-// np nodes per compute thread, 1 << stages_log2 shared-memory stages.
+// Whether the row pipeline serves a box, and its CTA shape: np nodes per
+// compute thread, 1 << stages_log2 shared-memory stages, work items in all
+// (rows; or, grouped, items of item.rows rows).
 struct RowPlan {
-    bool use = false;
+    bool use = false, grouped = false;
     int threads = 0;
     size_t smem = 0;
     int np = 1;
     uint32_t stages_log2 = 1;
+    uint64_t work = 0;
+    RowItems item{1, 1};
 };
+
 template <typename S>
-inline RowPlan row_plan(uint32_t nx)
+inline RowPlan row_plan(uint32_t nx, uint32_t ny, uint32_t nz)
 {
     RowPlan p;
     if (nx % 32 != 0 || nx < 32) return p;
     const size_t sb = row_stage_bytes<S>(nx);
     uint32_t cmax = kRowCompute;
-    // pairs from rows of 256 nodes (a full CTA of 4 compute warps); narrower
-    // rows run faster with one node per thread (measured at 128^3)
+    p.work = uint64_t(ny) * nz;
     const size_t cta_smem = kRowPairSmSmem / size_t(row_pair_ctas<S>());
-    if (!std::is_same<S, double>::value && row_pairs_enabled() && nx >= 2 * kRowPairCompute &&
-        2 * sb <= cta_smem) {
+    if (!std::is_same<S, double>::value && row_pairs_enabled() && 2 * nx <= kItemNodes) {
+        p.use = p.grouped = true;
+        p.np = 2;
+        p.smem = 2 * row_stage_bytes<S>(kItemNodes);
+        p.threads = kRowPairCompute + 32;
+        p.item.rows = std::min(kItemNodes / nx, ny);
+        p.item.per_plane = (ny + p.item.rows - 1) / p.item.rows;
+        p.work = uint64_t(p.item.per_plane) * nz;
+        return p;
+    }
+    if (!std::is_same<S, double>::value && row_pairs_enabled() && 2 * sb <= cta_smem) {
         p.np = 2;
         p.stages_log2 = (size_t(kRowMaxStages) * sb <= cta_smem) ? 2 : 1;
         cmax = kRowPairCompute;
@@ -1259,11 +1439,51 @@ inline RowPlan row_plan(uint32_t nx)
     return p;
 }
 
+// Launch of k_step_items for plan rp (rp.grouped), and its resident CTAs per
+// SM (also opts the kernels into their shared memory).
+template <typename S, typename R, int SC>
+cudaError_t launch_items_t(S *g, const StepArgs<R> &a, const RowPlan &rp, bool odd, bool stats, int grid,
+                           cudaStream_t s)
+{
+#define FLBM_LAUNCH_ITEMS(OD, ST) k_step_items<S, R, SC, OD, ST><<<grid, rp.threads, rp.smem, s>>>(g, a, rp.item)
+    if (odd) { if (stats) FLBM_LAUNCH_ITEMS(true, true); else FLBM_LAUNCH_ITEMS(true, false); }
+    else     { if (stats) FLBM_LAUNCH_ITEMS(false, true); else FLBM_LAUNCH_ITEMS(false, false); }
+#undef FLBM_LAUNCH_ITEMS
+    return cudaGetLastError();
+}
+template <typename S, typename R, int SC>
+int items_resident_t(const RowPlan &rp)
+{
+    const int dmax = int(kRowMaxSmem);
+    cudaFuncSetAttribute(k_step_items<S, R, SC, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dmax);
+    cudaFuncSetAttribute(k_step_items<S, R, SC, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dmax);
+    cudaFuncSetAttribute(k_step_items<S, R, SC, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dmax);
+    cudaFuncSetAttribute(k_step_items<S, R, SC, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dmax);
+    int nb = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_items<S, R, SC, true, true>,
+                                                                        rp.threads, rp.smem);
+    return e == cudaSuccess && nb > 0 ? nb : 0;
+}
+template <typename S, typename R>
+cudaError_t launch_items(S *g, const StepArgs<R> &a, const RowPlan &rp, int scheme, bool odd, bool stats, int grid,
+                         cudaStream_t s)
+{
+    if (scheme == 0) return launch_items_t<S, R, 0>(g, a, rp, odd, stats, grid, s);
+    if (scheme == 1) return launch_items_t<S, R, 1>(g, a, rp, odd, stats, grid, s);
+    return launch_items_t<S, R, 2>(g, a, rp, odd, stats, grid, s);
+}
+template <typename S, typename R>
+int items_resident(const RowPlan &rp, int scheme)
+{
+    return scheme == 0 ? items_resident_t<S, R, 0>(rp) : scheme == 1 ? items_resident_t<S, R, 1>(rp)
+                                                                     : items_resident_t<S, R, 2>(rp);
+}
+
 // One launch of the row kernel variant that plan rp picks.
 template <typename S, typename R, int SC, bool OD, bool ST>
 void launch_rows(S *g, const StepArgs<R> &a, const RowPlan &rp, int row_grid, cudaStream_t s)
 {
-    if constexpr (!std::is_same<S, double>::value) {
+    if constexpr (sizeof(S) == 2) {   // FP32: rows_paced
         if (rp.np == 2) {
             k_step_rows<S, R, SC, OD, ST, 2><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2);
             return;
@@ -1306,8 +1526,8 @@ template <typename S, typename R, typename I>
 cudaError_t launch_step_t(S *g, const StepArgs<R> &a, int scheme, bool odd, bool stats, int grid,
                           int row_grid, cudaStream_t s)
 {
-    const RowPlan rp = row_plan<S>(a.nx);
-    if (rp.use && row_grid > 0) {
+    const RowPlan rp = row_plan<S>(a.nx, a.ny, a.nz);
+    if (rp.use && !rp.grouped && row_grid > 0) {
 #define FLBM_LAUNCH_ROWS(SC, OD, ST) launch_rows<S, R, SC, OD, ST>(g, a, rp, row_grid, s)
         if (scheme == 0) {
             if (odd) { if (stats) FLBM_LAUNCH_ROWS(0, true, true); else FLBM_LAUNCH_ROWS(0, true, false); }
@@ -1356,12 +1576,12 @@ int prepare_rows(const RowPlan &rp, bool stats)
     return (e == cudaSuccess && nb > 0) ? nb : 0;
 }
 
-// Whether a box of row length nx runs the PACED two-node row kernel under
-// plan rp: FP32 storage, two nodes per thread, two stages.
+// Whether a box runs the PACED two-node row kernel under plan rp: FP32
+// storage, two nodes per thread, a row per item (288-512 nodes, two stages).
 template <typename S>
 inline bool rows_paced(const RowPlan &rp)
 {
-    return std::is_same<S, float>::value && rp.use && rp.np == 2 && rp.stages_log2 == 1;
+    return std::is_same<S, float>::value && rp.use && rp.np == 2 && !rp.grouped;
 }
 
 // Whether a box of row length nx runs the fixed-length two-node row kernel
@@ -1379,7 +1599,7 @@ template <typename S, typename R, uint32_t NXC, bool PACED = false>
 cudaError_t launch_rows_fixed(S *g, const StepArgs<R> &a, int scheme, bool odd, bool stats, int row_grid,
                               cudaStream_t s)
 {
-    const RowPlan rp = row_plan<S>(a.nx);
+    const RowPlan rp = row_plan<S>(a.nx, a.ny, a.nz);
 #define FLBM_LAUNCH_FIXED(SC, OD, ST) \
     k_step_rows<S, R, SC, OD, ST, 2, NXC, PACED><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2)
     if (scheme == 0) {
@@ -1398,9 +1618,8 @@ cudaError_t launch_rows_fixed(S *g, const StepArgs<R> &a, int scheme, bool odd, 
 
 // prepare_rows for the fixed-length or PACED kernels of one scheme (rows of nx).
 template <typename S, typename R, uint32_t NXC, bool PACED = false>
-int prepare_rows_fixed(int scheme, bool stats, uint32_t nx = NXC)
+int prepare_rows_fixed(int scheme, bool stats, const RowPlan &rp)
 {
-    const RowPlan rp = row_plan<S>(nx);
     if (scheme == 0) return prepare_rows<S, R, 0, 2, NXC, PACED>(rp, stats);
     if (scheme == 1) return prepare_rows<S, R, 1, 2, NXC, PACED>(rp, stats);
     return prepare_rows<S, R, 2, 2, NXC, PACED>(rp, stats);
@@ -1418,38 +1637,39 @@ int direct_resident(const DirectPlan &dp, bool stats)
     return e == cudaSuccess && nb > 0 ? nb : 1;
 }
 
-// The step kernels of a box of n nodes in rows of nx: the direct kernel's
+// The step kernels of a box: the direct kernel's
 // CTAs in all and resident per SM, and the row kernel's per SM (0 when the
 // row pipeline does not serve the box); also opts the row kernels into their
 // shared memory on the current device.
 template <typename S, typename R, typename I, int SC>
-void prepare_scheme(uint32_t nx, uint64_t n, bool stats, StepShape &shape)
+void prepare_scheme(uint32_t nx, uint32_t ny, uint32_t nz, bool stats, StepShape &shape)
 {
-    const DirectPlan dp = direct_plan<S>(n);
+    const DirectPlan dp = direct_plan<S>(uint64_t(nx) * ny * nz);
     shape.ctas = dp.ctas;
     shape.rows = 0;
     if constexpr (std::is_same<S, double>::value) shape.direct = direct_resident<S, R, I, SC, 1>(dp, stats);
     else shape.direct = dp.np == 2 ? direct_resident<S, R, I, SC, 2>(dp, stats) : direct_resident<S, R, I, SC, 1>(dp, stats);
-    const RowPlan rp = row_plan<S>(nx);
-    if (!rp.use) return;
+    const RowPlan rp = row_plan<S>(nx, ny, nz);
+    if (!rp.use || rp.grouped) return;   // grouped rows: the caller's translation unit
+    shape.work = rp.work;
     // the attribute is per kernel, shared by every context of the process:
     // set it to the largest staging any box may use, not to this box's
-    if constexpr (!std::is_same<S, double>::value) {
+    if constexpr (sizeof(S) == 2) {
         if (rp.np == 2) {
             shape.rows = prepare_rows<S, R, SC, 2>(rp, stats);
             return;
         }
     }
-    shape.rows = prepare_rows<S, R, SC, 1>(rp, stats);
+    if (rp.np == 1) shape.rows = prepare_rows<S, R, SC, 1>(rp, stats);
 }
 
 template <typename S, typename R, typename I>
-StepShape step_shape_t(int scheme, uint32_t nx, uint64_t n, bool stats)
+StepShape step_shape_t(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, bool stats)
 {
     StepShape shape;
-    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, n, stats, shape);
-    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, n, stats, shape);
-    else prepare_scheme<S, R, I, 2>(nx, n, stats, shape);
+    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, ny, nz, stats, shape);
+    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, ny, nz, stats, shape);
+    else prepare_scheme<S, R, I, 2>(nx, ny, nz, stats, shape);
     return shape;
 }
 
