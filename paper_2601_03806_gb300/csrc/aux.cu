@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch
 {
     __shared__ double red[kStatSlots * kStatTerms];   // at least kStatThreads
     static_assert(kStatSlots * kStatTerms >= kStatThreads, "the sums use it too");
+    __shared__ double tot[kStatSlots * NSTAT];
     __shared__ bool last;
     const int s = blockIdx.x, i = blockIdx.y, t = threadIdx.x;
     const double *p = f.partials + size_t(i) * f.slot_stride + s;
@@ -672,7 +673,9 @@ __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch
     __syncthreads();
     if (!last) return;
     __threadfence();
-    stats_update(st, f.totals, int(gridDim.y), f.step, n, red);
+    for (int e = t; e < int(gridDim.y) * NSTAT; e += kStatThreads) tot[e] = __ldcg(f.totals + e);   // other SMs' too
+    __syncthreads();
+    stats_update(st, tot, int(gridDim.y), f.step, n, red);
     if (t == 0) *f.arrived = 0u;
 }
 

@@ -651,8 +651,9 @@ int flbm_stats(flbm_ctx *c, flbm_stats_t *out)
     if (!c) return fail(nullptr, FLBM_E_INVALID, "ctx is NULL");
     if (!out) return fail(c, FLBM_E_INVALID, "out is NULL");
     DevStats h;
-    CK(c, cudaMemcpyAsync(&h, c->dstats, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    if (!c->host_stats) CK(c, cudaMemcpyAsync(&h, c->dstats, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
+    if (c->host_stats) h = *c->host_stats;   // written by the ensemble's kernels
     std::memset(out, 0, sizeof(*out));
     const double N = double(c->n);
     out->step = h.nsamp ? h.step : -1;
@@ -681,6 +682,7 @@ int flbm_stats_reset(flbm_ctx *c)
     if (!c) return fail(nullptr, FLBM_E_INVALID, "ctx is NULL");
     CK(c, cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
+    if (c->host_stats) std::memset(c->host_stats, 0, sizeof(DevStats));
     return FLBM_OK;
 }
 

@@ -64,6 +64,7 @@ struct flbm_ctx {
     // with it; its state may be replaced only while the ensemble's storage
     // is in the natural form
     flbm_ensemble *ens = nullptr;
+    flbm::DevStats *host_stats = nullptr;   // the ensemble's host copy of dstats (not owned)
     // FLBM_LEARNED: the network image on the device (flbm_set_mlp)
     unsigned char *mlp_img = nullptr;
     // FLBM_STATE_MOMENTS: two arrays of kMsVals * n floats; ms[ms_cur] holds

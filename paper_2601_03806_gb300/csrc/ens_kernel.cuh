@@ -249,8 +249,8 @@ __global__ void __maxnreg__(NP == 2 ? 168 : 112) k_step_ens(const __grid_constan
             const uint64_t i = begin + k;
             ens_advance(reps, a.nrep, i, r);
             const EnsReplica &rp = reps[r];
-            const EnsView<R> v{a.rk, step, rp.ctr2, rp.noise_rho0, R(rp.rho0), R(rp.sqrt_rho0),
-                               R(rp.lambda), R(rp.omega), R(rp.amp_h), R(rp.amp_g), a.flag, rp.bad_step};
+            const EnsView<R> v{a.rk, step, rp.ctr2, rp.noise_rho0, rp.rho0, rp.sqrt_rho0,
+                               rp.lambda, rp.omega, rp.amp_h, rp.amp_g, a.flag, rp.bad_step};
             const uint32_t nx = rp.nx, item_nodes = rp.item_nodes;
             uint32_t z, y0;
             ens_item(rp, i, z, y0);
@@ -364,18 +364,28 @@ __global__ void k_ens_post(const __grid_constant__ EnsArgs a, uint32_t cwarps, u
                            unsigned long long *dstep)
 {
     if (STATS) {
-        __shared__ double tot[NSTAT];
+        __shared__ double tot[NSTAT], mean[kStatTerms];
+        const long long step = (long long)(*dstep);
         const uint32_t r = blockIdx.x;
         const EnsReplica &rp = a.reps[r];
         if (threadIdx.x < NSTAT) {
             double t = 0.0;
-            for (int b = rp.cta_lo; b <= rp.cta_hi; ++b)
-                for (uint32_t w = 0; w < cwarps; ++w)
-                    t += a.partials[((size_t(b) + r) * kEnsMaxWarps + w) * NSTAT + threadIdx.x];
+            for (int b = rp.cta_lo; b <= rp.cta_hi; ++b) {
+                const double *p = a.partials + (size_t(b) + r) * kEnsMaxWarps * NSTAT + threadIdx.x;
+#pragma unroll 4
+                for (uint32_t w = 0; w < cwarps; ++w) t += p[w * NSTAT];
+            }
             tot[threadIdx.x] = t;
         }
         __syncthreads();
-        if (threadIdx.x == 0) stats_update(rp.st, tot, (long long)(*dstep), double(rp.n));
+        stats_update(rp.st, tot, 1, &step, double(rp.n), mean);
+        // a copy for the host, which then needs no transfer per replica to
+        // read them (328 of them took 6 ms)
+        __syncthreads();
+        static_assert(sizeof(DevStats) % 8 == 0, "copied in 8-byte words");
+        for (uint32_t w = threadIdx.x; w < sizeof(DevStats) / 8; w += 32)
+            reinterpret_cast<unsigned long long *>(rp.host_st)[w] =
+                reinterpret_cast<const volatile unsigned long long *>(rp.st)[w];
     }
     if (threadIdx.x == 0) {
         __threadfence();

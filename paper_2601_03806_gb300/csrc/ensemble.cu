@@ -38,6 +38,7 @@ struct flbm_ensemble {
     std::vector<size_t> offsets;        // byte offset of each replica in g
     std::vector<EnsReplica> htab;
     EnsReplica *dtab = nullptr;
+    DevStats *host_stats = nullptr;     // [nrep] copies of the accumulators (pinned, mapped)
     double *partials = nullptr;
     size_t partial_elems = 0;
     // device bookkeeping: [0] step counter, [1] post-kernel arrivals (low
@@ -297,6 +298,9 @@ int reset_all(flbm_ensemble *e)
         c->step = 0;
         c->phase = 0;
     }
+    // steps in flight (the autotuner's) write the copies too
+    ECK(e, cudaStreamSynchronize(e->stream));
+    std::memset(e->host_stats, 0, size_t(e->nrep) * sizeof(DevStats));
     ECK(e, cudaMemsetAsync(e->dbook, 0, 2 * sizeof(unsigned long long), e->stream));
     int rc = reset_flags(e);
     if (rc) return rc;
@@ -318,6 +322,7 @@ void release(flbm_ensemble *e)
     cudaFree(e->partials);
     cudaFree(e->dtab);
     cudaFree(e->dbook);
+    cudaFreeHost(e->host_stats);
     cudaFree(e->g);
     if (e->own_stream && e->stream) cudaStreamDestroy(e->stream);
     delete e;
@@ -376,6 +381,12 @@ int flbm_ensemble_create(const flbm_params *params, int count, void *cuda_stream
     err = cudaMalloc(&e->g, e->g_bytes);
     if (err == cudaSuccess) err = cudaMalloc(&e->dtab, size_t(count) * sizeof(EnsReplica));
     if (err == cudaSuccess) err = cudaMalloc(&e->dbook, (3 + size_t(count)) * sizeof(unsigned long long));
+    DevStats *mapped = nullptr;
+    if (err == cudaSuccess)
+        err = cudaHostAlloc(reinterpret_cast<void **>(&e->host_stats), size_t(count) * sizeof(DevStats),
+                            cudaHostAllocMapped);
+    if (err == cudaSuccess)
+        err = cudaHostGetDevicePointer(reinterpret_cast<void **>(&mapped), e->host_stats, 0);
     if (err != cudaSuccess) {
         e->err = std::string("cudaMalloc: ") + cudaGetErrorString(err);
         return bail(FLBM_E_NOMEM);
@@ -407,13 +418,15 @@ int flbm_ensemble_create(const flbm_params *params, int count, void *cuda_stream
         rp.nz = uint32_t(params[r].nz);
         rp.ctr2 = sa.ctr2;
         rp.noise_rho0 = sa.noise_rho0;
-        rp.rho0 = sa.rho0;
-        rp.sqrt_rho0 = sa.sqrt_rho0;
-        rp.lambda = sa.lambda;
-        rp.omega = sa.omega;
-        rp.amp_h = sa.amp_h;
-        rp.amp_g = sa.amp_g;
+        rp.rho0 = float(sa.rho0);
+        rp.sqrt_rho0 = float(sa.sqrt_rho0);
+        rp.lambda = float(sa.lambda);
+        rp.omega = float(sa.omega);
+        rp.amp_h = float(sa.amp_h);
+        rp.amp_g = float(sa.amp_g);
         rp.st = c->dstats;
+        rp.host_st = mapped + r;
+        c->host_stats = e->host_stats + r;
         rp.bad_step = e->bad_steps() + r;
     }
     // FLBM_INJECT_STARVE=1 (environment, failure-injection tests only): the

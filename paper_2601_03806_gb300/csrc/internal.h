@@ -86,10 +86,12 @@ struct EnsReplica {
     uint32_t items_per_plane;     // ny / rpi
     uint32_t ctr2;                // noise stream << 8
     int32_t noise_rho0;
-    double rho0, sqrt_rho0;       // the scalars of StepArgs, per replica
-    double lambda, omega, amp_h, amp_g;
+    // the scalars of StepArgs, per replica, in the kernels' FP32 (every item
+    // reads them; conversions from FP64 would run at two per clock and SM)
+    float rho0, sqrt_rho0, lambda, omega, amp_h, amp_g;
     int32_t cta_lo, cta_hi;       // CTAs whose chunks meet this replica
     DevStats *st;                 // accumulators of the replica's context
+    DevStats *host_st;            // their copy in host memory (mapped), written after each update
     unsigned long long *bad_step; // first unstable step of this replica
 };
 

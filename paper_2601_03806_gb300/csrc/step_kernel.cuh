@@ -1029,7 +1029,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // shared-memory access instead of an address computed per access.
 // PACED: the copy warp derives every copy's address from the row index
 // (row_segment_paced) instead of walking the rows (RowWalk): the same
-// addresses, issued more slowly.  Launched for the FP32 two-node rows (288-512 nodes; the HBM-bound 512^3 step), where walking made the step
+// addresses, issued more slowly.  Launched for the FP32 two-node rows
+// (288-512 nodes; the HBM-bound 512^3 step), where walking made the step
 // 1.5-2.1 % slower; in the other kernels walking is faster (512^3 FP16 +2.5
 // %).
 template <typename S, typename R, int SCHEME, bool ODD, bool STATS, int NP, uint32_t NXC = 0, bool PACED = false>
