@@ -198,7 +198,7 @@ void fill_constants_t(const flbm_params &p, StepArgs<R> &a)
 }
 
 template <typename R>
-StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr)
+StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr, bool chained = false)
 {
     StepArgs<R> a;
     std::memset(&a, 0, sizeof(a));
@@ -213,6 +213,7 @@ StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr)
     fill_constants_t<R>(c->p, a);
     a.tx_pad = c->tx_pad;
     a.normals = c->normals;
+    a.chained = chained;
     a.partials = partials;
     a.flag = &c->dflags->flag;
     a.bad_step = &c->dflags->bad_step;
@@ -557,6 +558,9 @@ int flbm_step(flbm_ctx *c, int64_t n)
             }
             CK(c, cudaEventRecord(c->ev[2 * c->ev_used], c->stream));
         }
+        // after the call's first step the stream's last work is this loop's own
+        // (events between the launches would be waited for)
+        const bool chained = s > 0 && !c->timing;
         double *const slot = c->partials + held * f.slot_stride;
         int reduced_grid = c->row_grid > 0 ? c->row_grid : c->grid;   // CTAs that wrote partials
         if (c->p.state_form == FLBM_STATE_MOMENTS) {
@@ -585,13 +589,13 @@ int flbm_step(flbm_ctx *c, int64_t n)
             e = launch_step_learned(static_cast<float *>(c->g), make_args<float>(c, t, slot), L, odd, stats, c->grid,
                                     c->stream);
         } else if (c->p.precision == FLBM_FP64)
-            e = launch_step_f64(static_cast<double *>(c->g), make_args<double>(c, t, slot), c->p.scheme, odd,
+            e = launch_step_f64(static_cast<double *>(c->g), make_args<double>(c, t, slot, chained), c->p.scheme, odd,
                                 stats, c->grid, c->row_grid, c->stream);
         else if (c->p.precision == FLBM_FP32)
-            e = launch_step_f32(static_cast<float *>(c->g), make_args<float>(c, t, slot), c->p.scheme, odd,
+            e = launch_step_f32(static_cast<float *>(c->g), make_args<float>(c, t, slot, chained), c->p.scheme, odd,
                                 stats, c->grid, c->row_grid, c->stream);
         else
-            e = launch_step_f16(c->g, make_args<float>(c, t, slot), c->p.scheme, odd, stats, c->grid,
+            e = launch_step_f16(c->g, make_args<float>(c, t, slot, chained), c->p.scheme, odd, stats, c->grid,
                                 c->row_grid, c->stream);
         if (e != cudaSuccess) {
             form_totals();   // of the steps that did run

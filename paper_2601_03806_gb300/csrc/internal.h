@@ -45,6 +45,8 @@ struct StepArgs {
     int32_t noise_rho0;           // phi_k uses rho0 instead of rho(x,t)
     uint32_t tx_pad;              // failure injection: bytes the row pipeline
                                   // expects beyond what it copies (0 normally)
+    uint32_t chained;             // host: the stream's last work is a step kernel or the totals of
+                                  // steps, and this launch may overlap its end (launch_step)
     R rho0;
     R sqrt_rho0;
     // Relaxation and noise scalars; the per-mode factors (syn_scale,

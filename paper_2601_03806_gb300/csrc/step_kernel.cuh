@@ -641,6 +641,33 @@ __device__ __forceinline__ void collide_core(V (&v)[3][3][3], const A &a,
 }
 
 // ---------------------------------------------------------------------------
+// Consecutive steps as dependent launches: a step kernel lets its successor
+// be launched as soon as all its CTAs run, and itself touches global memory
+// only after its predecessor has finished, so the launch of step t + 1 and its
+// set-up (barriers, index arithmetic) overlap the last CTAs of step t: 16^3
+// FP32 8.0 -> 5.1 us a step, 64^3 18.3 -> 16.2, 128^3 83.2 -> 82.0.  Without
+// the launch attribute both instructions do nothing.
+__device__ __forceinline__ void step_ready() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void step_started() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_step(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t s, bool chained,
+                        Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // k_step: direct loads/stores (general boxes)
 
 // Periodic neighbour offsets of node (x,y,z): xs[d], ry[d], rz[d] for the
@@ -791,6 +818,8 @@ __global__ void __launch_bounds__(kBlock, NP == 2 ? 3 : FLBM_MIN_BLOCKS) k_step(
             cp_async_commit();
         }
     };
+    step_started();
+    step_ready();
     stage(n);
     uint32_t it = 0;
     for (uint64_t base = n - threadIdx.x; base < a.n; base += stride, n += stride, ++it) {
@@ -1064,6 +1093,8 @@ __global__ void __launch_bounds__(NP == 2 ? kRowPairCompute + 32 : kRowCompute +
     }
     if (STATS) totals_init(tot);
     __syncthreads();
+    step_started();
+    step_ready();
 
     if (threadIdx.x >= nc) {
         // ---------------- producer warp ----------------
@@ -1262,6 +1293,8 @@ __global__ void __launch_bounds__(kRowPairCompute + 32, row_pair_ctas<S>())
     }
     if (STATS) totals_init(tot);
     __syncthreads();
+    step_started();
+    step_ready();
     auto rows_of = [&](uint32_t y0) { return min(items.rows, a.ny - y0); };
 
     if (threadIdx.x >= nc) {
@@ -1446,7 +1479,8 @@ template <typename S, typename R, int SC>
 cudaError_t launch_items_t(S *g, const StepArgs<R> &a, const RowPlan &rp, bool odd, bool stats, int grid,
                            cudaStream_t s)
 {
-#define FLBM_LAUNCH_ITEMS(OD, ST) k_step_items<S, R, SC, OD, ST><<<grid, rp.threads, rp.smem, s>>>(g, a, rp.item)
+#define FLBM_LAUNCH_ITEMS(OD, ST) \
+    launch_step(k_step_items<S, R, SC, OD, ST>, grid, rp.threads, rp.smem, s, a.chained, g, a, rp.item)
     if (odd) { if (stats) FLBM_LAUNCH_ITEMS(true, true); else FLBM_LAUNCH_ITEMS(true, false); }
     else     { if (stats) FLBM_LAUNCH_ITEMS(false, true); else FLBM_LAUNCH_ITEMS(false, false); }
 #undef FLBM_LAUNCH_ITEMS
@@ -1486,11 +1520,12 @@ void launch_rows(S *g, const StepArgs<R> &a, const RowPlan &rp, int row_grid, cu
 {
     if constexpr (sizeof(S) == 2) {   // FP32: rows_paced
         if (rp.np == 2) {
-            k_step_rows<S, R, SC, OD, ST, 2><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2);
+            launch_step(k_step_rows<S, R, SC, OD, ST, 2>, row_grid, rp.threads, rp.smem, s, a.chained, g, a,
+                        rp.stages_log2);
             return;
         }
     }
-    k_step_rows<S, R, SC, OD, ST, 1><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2);
+    launch_step(k_step_rows<S, R, SC, OD, ST, 1>, row_grid, rp.threads, rp.smem, s, a.chained, g, a, rp.stages_log2);
 }
 
 template <typename S, typename R, typename I, int SC, bool OD, bool ST, typename Plan>
@@ -1498,11 +1533,11 @@ void launch_direct(S *g, const StepArgs<R> &a, const Plan &dp, int grid, cudaStr
 {
     if constexpr (!std::is_same<S, double>::value) {
         if (dp.np == 2) {
-            k_step<S, R, I, SC, OD, ST, 2><<<grid, dp.threads, 0, s>>>(g, a);
+            launch_step(k_step<S, R, I, SC, OD, ST, 2>, grid, dp.threads, 0, s, a.chained, g, a);
             return;
         }
     }
-    k_step<S, R, I, SC, OD, ST, 1><<<grid, dp.threads, 0, s>>>(g, a);
+    launch_step(k_step<S, R, I, SC, OD, ST, 1>, grid, dp.threads, 0, s, a.chained, g, a);
 }
 
 // Shape of the direct kernel for a box of n nodes: nodes and threads per CTA.
@@ -1602,7 +1637,8 @@ cudaError_t launch_rows_fixed(S *g, const StepArgs<R> &a, int scheme, bool odd, 
 {
     const RowPlan rp = row_plan<S>(a.nx, a.ny, a.nz);
 #define FLBM_LAUNCH_FIXED(SC, OD, ST) \
-    k_step_rows<S, R, SC, OD, ST, 2, NXC, PACED><<<row_grid, rp.threads, rp.smem, s>>>(g, a, rp.stages_log2)
+    launch_step(k_step_rows<S, R, SC, OD, ST, 2, NXC, PACED>, row_grid, rp.threads, rp.smem, s, a.chained, g, a, \
+                rp.stages_log2)
     if (scheme == 0) {
         if (odd) { if (stats) FLBM_LAUNCH_FIXED(0, true, true); else FLBM_LAUNCH_FIXED(0, true, false); }
         else     { if (stats) FLBM_LAUNCH_FIXED(0, false, true); else FLBM_LAUNCH_FIXED(0, false, false); }
