@@ -350,13 +350,13 @@ __device__ __forceinline__ void normal_pair(uint32_t w1, uint32_t w2, float &rad
     rad = __fmul_rn(t, rsqrtf(t));
     __sincosf(__fmaf_rn(u2, 6.2831853071795865f, -3.1415926535897932f), &sa, &ca);
 }
-// FP64: from tables (normal_tab.cuh), 32 FP64 operations a pair instead of
-// about 75 with the library's log and sincospi; the FP64 pipe bounds the
+// FP64: from tables (normal_tab.cuh), 29 FP64 operations a pair instead of
+// about 75 with the library's log, sqrt and sincospi; the FP64 pipe bounds the
 // FP64 step (86 % busy; 1350 operations a node before).
 __device__ __forceinline__ void normal_pair(const NormalTab &tab, uint32_t w1, uint32_t w2, double &rad, double &ca,
                                             double &sa)
 {
-    rad = sqrt(neg2_log(tab, w1 >> 9));
+    rad = sqrt_normal(neg2_log(tab, w1 >> 9));
     neg_cos_sin(tab, w2 >> 9, ca, sa);
 }
 // Two nodes, one per lane (words of node a in .x, of node b in .y).
@@ -406,6 +406,29 @@ __host__ __device__ constexpr double noise_scale(int mk)
            sqrt_b_over_cs2(mode_deg(mk) % 3, (mode_deg(mk) / 3) % 3, mode_deg(mk) / 9);
 }
 
+// The same scale as a function of how many of the mode's degrees are 1 and 2,
+// so that modes of one kind share one constant to the last bit (FP64).
+__host__ __device__ constexpr double noise_scale_of_kind(int mk)
+{
+    const int d[3] = {mode_deg(mk) % 3, (mode_deg(mk) / 3) % 3, mode_deg(mk) / 9};
+    double s = -1.7320508075688772935;
+    for (int g = 0; g < 3; ++g)
+        for (int a = 0; a < 3; ++a)
+            if (d[a] == g) s *= kappa1d(g) * sqrt_beta1d(g);
+    return s;
+}
+
+// Scaled normals: m-th of a block of modes, from its radius and cosine or
+// sine.  FP32: in the reconstruction's units, so that only the amplitude is
+// left; FP64: without the mode's scale, which noise_synthesise multiplies into
+// the amplitude once per kind of mode instead of once per mode.
+template <typename V>
+__device__ __forceinline__ V scaled_normal(V rad, V trig, int mk)
+{
+    if constexpr (std::is_same<V, double>::value) return vmul(rad, trig);
+    else return vmul(vmul(rad, vset<V>(noise_scale(mk))), trig);
+}
+
 // A is the step's scalar set: StepArgs<R> for one box, or a per-replica view
 // with the same member names (rk, step, ctr2, rho0, ...) for an ensemble.
 template <typename V, typename A>
@@ -419,7 +442,7 @@ __device__ __forceinline__ void draw_noise(const A &a, uint32_t node, V (&nz)[kN
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             const int mk = 4 + 4 * blk + m;
-            if (mk < kQ) nz[mk - 4] = vmul(vmul(m < 2 ? rad0 : rad1, vset<V>(noise_scale(mk))), trig[m]);
+            if (mk < kQ) nz[mk - 4] = scaled_normal(m < 2 ? rad0 : rad1, trig[m], mk);
         }
     }
 }
@@ -535,7 +558,9 @@ __device__ __forceinline__ void collide_modes(V (&v)[3][3][3], const A &a, V (&a
                     q = vmul(v[i][j][k], syn);                  // momentum, conserved
                 } else if (ord == 2 || SCHEME == 2) {
                     const V aeq = aeq_coef(i, j, k, jj, uu);
-                    if (ord == 2)   // a_eq + (1 - omega)(m - a_eq) = omega a_eq + lambda m
+                    if (ord == 2 && std::is_same<V, double>::value)   // three operations for five
+                        q = vfma(vmul(lam, vmul(syn, unfwd)), v[i][j][k], vmul(vmul(syn, om), aeq));
+                    else if (ord == 2)   // a_eq + (1 - omega)(m - a_eq) = omega a_eq + lambda m
                         q = vmul(syn, vfma(lam, vmul(v[i][j][k], unfwd), vmul(om, aeq)));
                     else            // Reg ghosts: a_eq (unit relaxation)
                         q = vmul(syn, aeq);
@@ -563,12 +588,19 @@ __device__ __forceinline__ void noise_synthesise(V (&qm)[3][3][3], V rho, const 
     {
         const V sr = a.noise_rho0 ? vbc(a.sqrt_rho0, rho) : sqrt_(rho);
         const V sh = vmul(sr, vbc(a.amp_h, rho)), sg = vmul(sr, vbc(a.amp_g, rho));
+        // amplitude of mode mk (FP64: times its scale, which depends on how
+        // many of its degrees are 1 and 2: the compiler forms each once)
+        auto amp = [&](int mk) {
+            const V s = mk <= 9 ? sh : sg;
+            if constexpr (std::is_same<V, double>::value) return vmul(s, vset<V>(noise_scale_of_kind(mk)));
+            else return s;
+        };
         if (PREDRAWN) {
 #pragma unroll
             for (int mk = 4; mk < kQ; ++mk) {
                 const int d = mode_deg(mk);
                 V &q = qm[d % 3][(d / 3) % 3][d / 9];
-                q = vfma(mk <= 9 ? sh : sg, nz[mk - 4], q);
+                q = vfma(amp(mk), nz[mk - 4], q);
             }
         } else {
             // pairs never mix hydrodynamic and ghost modes
@@ -583,9 +615,9 @@ __device__ __forceinline__ void noise_synthesise(V (&qm)[3][3][3], V rho, const 
                     if (mk < kQ) {
                         const int d = mode_deg(mk);
                         // same rounding order as draw_noise + the PREDRAWN branch
-                        const V t = vmul(vmul(m < 2 ? rad0 : rad1, vset<V>(noise_scale(mk))), trig[m]);
+                        const V t = scaled_normal(m < 2 ? rad0 : rad1, trig[m], mk);
                         V &q = qm[d % 3][(d / 3) % 3][d / 9];
-                        q = vfma(mk <= 9 ? sh : sg, t, q);
+                        q = vfma(amp(mk), t, q);
                     }
                 }
             }
