@@ -158,6 +158,9 @@ cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool 
 // Nodes from which the direct kernel takes two per thread in CTAs of kBlock
 // threads (below, one per thread in CTAs of a warp).
 constexpr uint64_t kDirectPairs = 65536;
+// FP64 nodes up to which an SM's warps share 32 of them (k_step_few; 152 SMs);
+// larger boxes keep the FP64 units busy with a warp per 32 nodes.
+constexpr uint64_t kDirectFew = 4864;
 // Launch shape of the step kernels for a box: the direct kernel's CTAs and how many of them an SM holds, and the row
 // pipeline's CTAs per SM (0 when it does not serve rows of length nx); the
 // slab stride ns picks the index width.  Also prepares the kernels'

@@ -912,6 +912,79 @@ __global__ void __launch_bounds__(kBlock, NP == 2 ? 3 : FLBM_MIN_BLOCKS) k_step(
     }
 }
 
+// The direct FP64 step of a box of at most a warp of nodes per SM.  An FP64
+// instruction of a warp holds its sub-partition's unit for 64 cycles, whatever
+// its lanes and dependencies, so one warp that draws, projects, collides and
+// reconstructs takes 64 times its 800 operations.  A CTA of 32 nodes instead
+// spreads them over an SM's four sub-partitions: six warps (two on each of
+// three) draw one Philox block of four normals each into shared memory while
+// the last, alone on the fourth, loads the nodes and projects them; then it
+// adds the noise and reconstructs.  Its shared memory keeps a CTA to an SM: a
+// second one, placed while the step before still ran, would double the time.
+// 16^3: 20 us a step, 30 with one warp doing all of it.
+constexpr int kFewThreads = 8 * 32;
+constexpr uint32_t kFewCollide = 7;   // the collision's warp; warp 3 of its sub-partition stays idle
+constexpr size_t kFewSmem = 120 * 1024;
+template <int SCHEME, bool ODD, bool STATS>
+__global__ void __launch_bounds__(kFewThreads, 1) k_step_few(double *__restrict__ g, const StepArgs<double> a)
+{
+    __shared__ TotSlot<double> tot[32][NSTAT];
+    __shared__ double normals[kNoise][32];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double acc[NSTAT];
+#pragma unroll
+    for (int s = 0; s < NSTAT; ++s) acc[s] = 0.0;
+    if (STATS) totals_init(tot);
+    __syncthreads();
+    step_started();
+    step_ready();
+    for (uint64_t base = uint64_t(blockIdx.x) * 32; base < a.n; base += uint64_t(gridDim.x) * 32) {
+        const uint64_t n = base + lane;
+        const bool on = n < a.n;
+        const NodeWalk w(a, on ? n : 0);
+        const Nbr<uint64_t> nb(w.x, w.y, w.z, a.nx, a.ny, a.nz);
+        double v[3][3][3], qm[3][3][3], rho = 1.0, dj[4];
+        if (warp != 3 && warp != kFewCollide) {
+            const int blk = int(warp < 3 ? warp : warp - 1);
+            double rad0, c0, s0, rad1, c1, s1;
+            block_normals(a, uint32_t(n), blk, rad0, c0, s0, rad1, c1, s1);
+            const int m0 = 4 * blk;   // of modes 4 + m0 ..
+            normals[m0][lane] = scaled_normal(rad0, c0, 4 + m0);
+            normals[m0 + 1][lane] = scaled_normal(rad0, s0, 5 + m0);
+            normals[m0 + 2][lane] = scaled_normal(rad1, c1, 6 + m0);
+            if (m0 + 3 < kNoise) normals[m0 + 3][lane] = scaled_normal(rad1, s1, 7 + m0);
+        } else if (warp == kFewCollide && on) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        v[i][j][k] = g[pop_index<uint64_t, ODD, true>(nb, n, a.ns, i, j, k)];
+            collide_modes<double, SCHEME, STATS>(v, a, acc, qm, rho, dj);
+        }
+        __syncthreads();
+        if (warp == kFewCollide && on) {
+            double nz[kNoise];
+#pragma unroll
+            for (int m = 0; m < kNoise; ++m) nz[m] = normals[m][lane];
+            noise_synthesise<double, true>(qm, rho, a, nz, uint32_t(n), v);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        g[pop_index<uint64_t, ODD, false>(nb, n, a.ns, i, j, k)] = v[i][j][k];
+        }
+        __syncthreads();   // the next nodes' normals reuse the buffer
+    }
+    if (STATS) {
+        warp_flush(acc, tot);   // only the collision's are not zero
+        block_store_totals(tot, a.partials + size_t(blockIdx.x) * NSTAT);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // k_step_rows: TMA bulk-copy row pipeline
 
@@ -1563,6 +1636,12 @@ void launch_rows(S *g, const StepArgs<R> &a, const RowPlan &rp, int row_grid, cu
 template <typename S, typename R, typename I, int SC, bool OD, bool ST, typename Plan>
 void launch_direct(S *g, const StepArgs<R> &a, const Plan &dp, int grid, cudaStream_t s)
 {
+    if constexpr (std::is_same<S, double>::value) {
+        if (dp.few) {
+            launch_step(k_step_few<SC, OD, ST>, grid, kFewThreads, kFewSmem, s, a.chained, g, a);
+            return;
+        }
+    }
     if constexpr (!std::is_same<S, double>::value) {
         if (dp.np == 2) {
             launch_step(k_step<S, R, I, SC, OD, ST, 2>, grid, dp.threads, 0, s, a.chained, g, a);
@@ -1578,6 +1657,7 @@ void launch_direct(S *g, const StepArgs<R> &a, const Plan &dp, int grid, cudaStr
 struct DirectPlan {
     int np, threads;
     uint64_t ctas;
+    bool few = false;   // k_step_few (FP64)
 };
 template <typename S>
 inline DirectPlan direct_plan(uint64_t n)
@@ -1585,6 +1665,7 @@ inline DirectPlan direct_plan(uint64_t n)
     DirectPlan p;
     p.np = !std::is_same<S, double>::value && row_pairs_enabled() && n >= kDirectPairs ? 2 : 1;
     p.threads = n >= kDirectPairs ? kBlock : 32;
+    p.few = std::is_same<S, double>::value && n <= kDirectFew;
     const uint64_t span = uint64_t(p.np) * p.threads;
     p.ctas = (n + span - 1) / span;
     return p;
@@ -1716,8 +1797,14 @@ void prepare_scheme(uint32_t nx, uint32_t ny, uint32_t nz, bool stats, StepShape
     const DirectPlan dp = direct_plan<S>(uint64_t(nx) * ny * nz);
     shape.ctas = dp.ctas;
     shape.rows = 0;
-    if constexpr (std::is_same<S, double>::value) shape.direct = direct_resident<S, R, I, SC, 1>(dp, stats);
-    else shape.direct = dp.np == 2 ? direct_resident<S, R, I, SC, 2>(dp, stats) : direct_resident<S, R, I, SC, 1>(dp, stats);
+    if constexpr (std::is_same<S, double>::value) {
+        const int sm = int(kFewSmem);
+        cudaFuncSetAttribute(k_step_few<SC, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_few<SC, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_few<SC, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_few<SC, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        shape.direct = dp.few ? 1 : direct_resident<S, R, I, SC, 1>(dp, stats);
+    } else shape.direct = dp.np == 2 ? direct_resident<S, R, I, SC, 2>(dp, stats) : direct_resident<S, R, I, SC, 1>(dp, stats);
     const RowPlan rp = row_plan<S>(nx, ny, nz);
     if (!rp.use || rp.grouped) return;   // grouped rows: the caller's translation unit
     shape.work = rp.work;

@@ -40,7 +40,8 @@ def test_two_nodes_per_thread_give_the_same_bits(F, monkeypatch, prec, shape):
         assert np.allclose(sa["u2"], sb["u2"], rtol=1e-5) and np.allclose(sa["m_var"], sb["m_var"], rtol=1e-4)
 
 
-@pytest.mark.parametrize("shape", [(37, 43, 61), (31, 1, 1), (33, 1, 1), (5, 13, 31)])
+# FP64: an SM's warps share 32 nodes up to 4,864
+@pytest.mark.parametrize("shape", [(37, 43, 61), (31, 1, 1), (33, 1, 1), (5, 13, 31), (19, 16, 16), (4865, 1, 1)])
 def test_against_the_oracle(F, oracle_mod, shape):
     nx, ny, nz = shape
     f0 = F.Lattice(nx, ny, nz, 0.8, 1e-4, seed=8)
