@@ -240,6 +240,12 @@ def strip_comments(src: str) -> str:
     return "\n".join(ln for ln in lines if ln)
 
 
+def total_launches(steps) -> int:
+    """Launches that form the reductions' totals in one call of `steps` steps
+    (16 reduced steps at a time)."""
+    return -(-int(steps) // 16)
+
+
 def kernel_source_hash(sources=None) -> str:
     """sha256 (first 16 hex digits) of the kernel sources, comments left out."""
     h = hashlib.sha256()
@@ -467,9 +473,14 @@ def run_ours(args, rank, local, ws):
     traffic = {"fp32": recorded_traffic(N),
                "fp16": recorded_traffic(N, TRAFFIC16_FILE, KERNEL16_SOURCES)}.get(args.precision)
     rows_path = nx % 32 == 0 and 2 * 27 * nx * es <= 200 * 1024 and os.environ.get("FLBM_ROWS", "1") != "0"
-    # two nodes per thread for FP32 / FP16 rows of 256 and more (FLBM_ROW_PAIRS=0: one)
-    pairs = (args.precision != "fp64" and nx >= 256 and 2 * 27 * nx * es <= 2 * 27 * 512 * 4
+    # small boxes run the direct kernel (FLBM_ROWS=1: the row pipeline at any size)
+    if N < (1 << (16 if args.precision == "fp64" else 19)) and os.environ.get("FLBM_ROWS") != "1":
+        rows_path = False
+    # two nodes per thread in FP32 / FP16 (FLBM_ROW_PAIRS=0: one), rows of up
+    # to 256 nodes in grouped work items
+    pairs = (args.precision != "fp64" and 2 * 27 * nx * es <= 2 * 27 * 512 * 4
              and os.environ.get("FLBM_ROW_PAIRS", "1") != "0")
+    grouped = rows_path and pairs and nx <= 256
     st_name = {"fp32": "float", "fp16": "__half", "fp64": "double"}[args.precision]
     # FP16 rows of exactly 512 nodes run the kernel with the row length fixed at compile time
     fixed = pairs and args.precision == "fp16" and nx == 512
@@ -479,6 +490,10 @@ def run_ours(args, rank, local, ws):
              % (st_name, 2 if pairs else 1, ",NXC=512" if fixed else (",PACED" if paced else ""),
                 "two nodes per thread" if pairs else "one node per thread")
              if rows_path else "flbm::k_step<%s,GMF,*,stats> (direct)" % st_name)
+    if grouped:
+        kname = ("flbm::k_step_items<%s,GMF,*,stats> (TMA row pipeline, grouped rows, two nodes per thread)"
+                 % st_name)
+        traffic = None     # the records are of the one-row items
     if rows_path and not pairs:
         traffic = None     # the records are of the two-node kernel
     if args.precision == "fp16" and not fixed:
@@ -565,7 +580,7 @@ def run_ours(args, rank, local, ws):
             "data": "synthetic", "config": workload_config(n, ws, args.precision, (nx, ny, nz), moments),
             "roofline": roofline,
             "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": int(launches) + int(args.steps),
+            "gpu_launches": int(launches) + total_launches(args.steps),
             "clocks": clk.summary(),
             "equipartition": {"u2_avg_over_kT_rho0": u2_ratio,
                               "max_abs_error": max(abs(x - 1) for x in u2_ratio),
@@ -1062,7 +1077,7 @@ def run_learned(args, rank, local, ws):
                        "l2": "inputs larger than L2 (%.2f GB state vs 129 MB L2)" % (108 * N / 1e9),
                        "parallelism": "replicas x%d" % ws},
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "plain_kernel": plain,
-            "gpu_launches": int(launches) + int(args.steps), "clocks": clocks,
+            "gpu_launches": int(launches) + total_launches(args.steps), "clocks": clocks,
             "training": training,
             "statistics": {"learned": stats_learned, "gmf": stats_gmf},
             "equipartition": {"u2_avg_over_kT_rho0": u2, "max_abs_error": max(abs(x - 1) for x in u2),
