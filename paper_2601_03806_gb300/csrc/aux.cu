@@ -652,7 +652,6 @@ __global__ void __launch_bounds__(kPairBlock) k_mlp_pairs(const S *__restrict__ 
 // CTAs per step because FP64 adds run at two per clock and SM: one CTA per
 // step took 15-17 us a step, a seventh of the 128^3 step and most of the 64^3
 // one; with the means' divisions in parallel this takes under 1 us a step.
-constexpr int kStatThreads = 128;
 __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch f, DevStats *st, double n)
 {
     __shared__ double red[kStatSlots * kStatTerms];   // at least kStatThreads
@@ -660,18 +659,9 @@ __global__ void __launch_bounds__(kStatThreads) k_stats_finalize(const StatBatch
     __shared__ double tot[kStatSlots * NSTAT];
     __shared__ bool last;
     const int s = blockIdx.x, i = blockIdx.y, t = threadIdx.x;
-    const double *p = f.partials + size_t(i) * f.slot_stride + s;
-    double v = 0.0;
-#pragma unroll 4
-    for (int b = t; b < f.nblocks[i]; b += kStatThreads) v += p[size_t(b) * NSTAT];
-    red[t] = v;
-    __syncthreads();
-    for (int w = kStatThreads / 2; w > 0; w >>= 1) {
-        if (t < w) red[t] += red[t + w];
-        __syncthreads();
-    }
+    const double sum = stat_total(f.partials + size_t(i) * f.slot_stride + s, f.nblocks[i], red);
     if (t == 0) {
-        f.totals[i * NSTAT + s] = red[0];
+        f.totals[i * NSTAT + s] = sum;
         __threadfence();
         last = atomicAdd(f.arrived, 1u) == gridDim.x * gridDim.y - 1;
     }

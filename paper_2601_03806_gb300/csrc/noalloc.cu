@@ -19,6 +19,7 @@
 #include "ctx.h"
 #include "internal.h"
 #include "lattice.cuh"
+#include "stats.cuh"
 
 namespace flbm {
 namespace {
@@ -57,26 +58,13 @@ cudaError_t scratch_address(int dev, NoallocScratch **out)
     return cudaSuccess;
 }
 
-// Fixed-order sum of the per-CTA partials into the caller's 13 doubles.
-__global__ void k_noalloc_sums(const NoallocScratch *sc, int nblocks, double *sums)
+// CTA s: sum s of the per-CTA partials into the caller's 13 doubles, in the
+// order of flbm_step's totals.
+__global__ void __launch_bounds__(kStatThreads) k_noalloc_sums(const NoallocScratch *sc, int nblocks, double *sums)
 {
-    __shared__ double red[NSTAT][256];
-    double loc[NSTAT];
-#pragma unroll
-    for (int s = 0; s < NSTAT; ++s) loc[s] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int s = 0; s < NSTAT; ++s) loc[s] += sc->partials[size_t(b) * NSTAT + s];
-#pragma unroll
-    for (int s = 0; s < NSTAT; ++s) red[s][threadIdx.x] = loc[s];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int s = 0; s < NSTAT; ++s) red[s][threadIdx.x] += red[s][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x < NSTAT) sums[threadIdx.x] = red[threadIdx.x][0];
+    __shared__ double red[kStatThreads];
+    const double t = stat_total(sc->partials + blockIdx.x, nblocks, red);
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
 }
 
 // Errors are reported through flbm_last_error(NULL), like create-time ones.
@@ -154,7 +142,7 @@ extern "C" int flbm_step_noalloc(const flbm_params *p, void *dev_state, int64_t 
     cudaError_t e = launch_step_f32(static_cast<float *>(dev_state), a, p->scheme, parity != 0, true,
                                     grid, row_grid, s);
     if (e == cudaSuccess) {
-        k_noalloc_sums<<<1, 256, 0, s>>>(sc, used, dev_sums);
+        k_noalloc_sums<<<NSTAT, kStatThreads, 0, s>>>(sc, used, dev_sums);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return noalloc_fail(FLBM_E_CUDA, cudaGetErrorString(e));

@@ -1,9 +1,30 @@
-// stats.cuh -- accumulation of reduced steps into DevStats (row a9).
+// stats.cuh -- totals of reduced steps and their accumulation into DevStats
+// (row a9).
 #pragma once
 
 #include "internal.h"
 
 namespace flbm {
+
+// The sum over nblocks CTAs of one of the NSTAT sums, p[0], p[NSTAT], ..., by
+// a CTA of kStatThreads threads in a fixed order (valid in thread 0): every
+// entry point's totals have the same bits.  red: kStatThreads doubles of
+// shared memory.
+constexpr int kStatThreads = 128;
+__device__ __forceinline__ double stat_total(const double *p, int nblocks, double *red)
+{
+    const int t = threadIdx.x;
+    double v = 0.0;
+#pragma unroll 4
+    for (int b = t; b < nblocks; b += kStatThreads) v += p[size_t(b) * NSTAT];
+    red[t] = v;
+    __syncthreads();
+    for (int w = kStatThreads / 2; w > 0; w >>= 1) {
+        if (t < w) red[t] += red[t + w];
+        __syncthreads();
+    }
+    return red[0];
+}
 
 // Adds `count` <= kStatSlots consecutive reduced steps to st, in order, by the
 // threads of a CTA (32 at least): totals[i][NSTAT], in shared memory, are the
