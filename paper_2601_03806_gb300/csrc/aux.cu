@@ -9,6 +9,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "error_free.cuh"
 #include "internal.h"
 #include "stats.cuh"
 #include "lattice.cuh"
@@ -344,41 +345,15 @@ __global__ void __launch_bounds__(256, 4) k_observable(const S *__restrict__ g, 
 // ---------------------------------------------------------------------------
 // Shell binning of the R2C spectrum [nz][ny][nx/2+1] (complex of T).
 
-// A sum of squares: FP32 spectra keep it as an exact-to-48-bits FP32 pair
-// (FP64 operations, two per clock and SM, bounded the kernel before: 84 % of
-// that pipe, 324 us at 256^3), FP64 spectra in FP64.
-template <typename T> struct ShellSum;
-template <> struct ShellSum<float> {
-    float hi, lo;
-    __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
-    __device__ __forceinline__ void add(float h, float l)
-    {
-        float e;
-        hi = two_sum(hi, h, e);
-        lo += e + l;
-    }
-    __device__ __forceinline__ void add(const ShellSum &o) { add(o.hi, o.lo); }
-    __device__ __forceinline__ void add_square(float v)
-    {
-        const float p = __fmul_rn(v, v);
-        add(p, __fmaf_rn(v, v, -p));
-    }
-    __device__ __forceinline__ void scale2() { hi *= 2.0f; lo *= 2.0f; }
-    __device__ __forceinline__ ShellSum up(int d) const
-    {
-        return ShellSum{__shfl_up_sync(0xffffffffu, hi, d), __shfl_up_sync(0xffffffffu, lo, d)};
-    }
-    __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
-};
-template <> struct ShellSum<double> {
-    double v;
-    __device__ __forceinline__ void zero() { v = 0.0; }
-    __device__ __forceinline__ void add(const ShellSum &o) { v += o.v; }
-    __device__ __forceinline__ void add_square(double x) { v = fma(x, x, v); }
-    __device__ __forceinline__ void scale2() { v *= 2.0; }
-    __device__ __forceinline__ ShellSum up(int d) const { return ShellSum{__shfl_up_sync(0xffffffffu, v, d)}; }
-    __device__ __forceinline__ double value() const { return v; }
-};
+__device__ __forceinline__ ShellSum<float> shell_up(const ShellSum<float> &v, int d)
+{
+    return ShellSum<float>{__shfl_up_sync(0xffffffffu, v.hi, d), __shfl_up_sync(0xffffffffu, v.mid, d),
+                           __shfl_up_sync(0xffffffffu, v.lo, d)};
+}
+__device__ __forceinline__ ShellSum<double> shell_up(const ShellSum<double> &v, int d)
+{
+    return ShellSum<double>{__shfl_up_sync(0xffffffffu, v.v, d)};
+}
 
 // Power of two that brings a spectrum whose field peaks at `peak` into a
 // range where FP32 squares neither overflow nor underflow: every amplitude is
@@ -406,10 +381,13 @@ __device__ __forceinline__ long long shell_of(unsigned long long n2)
 
 constexpr int kShellWarps = 8;
 constexpr size_t kShellSmem = 200 * 1024;
-// Warps of a CTA whose private bins (a sum and a count per shell) fit.
-inline int shell_warps(int nshell)
+// Bytes of a bin (a sum and a count), and warps of a CTA whose private bins fit.
+template <typename T>
+constexpr size_t kShellBin = sizeof(ShellSum<T>) + sizeof(unsigned int);
+template <typename T>
+int shell_warps(int nshell)
 {
-    const size_t w = kShellSmem / (size_t(nshell) * (sizeof(double) + sizeof(unsigned int)));
+    const size_t w = kShellSmem / (size_t(nshell) * kShellBin<T>);
     return w < size_t(kShellWarps) ? int(w) : kShellWarps;
 }
 
@@ -428,8 +406,7 @@ __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict
     extern __shared__ __align__(16) unsigned char shell_raw[];
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     ShellSum<T> *const sums = reinterpret_cast<ShellSum<T> *>(shell_raw);
-    unsigned int *const cnts = reinterpret_cast<unsigned int *>(shell_raw + size_t(warps) * nshell * sizeof(double));
-    static_assert(sizeof(ShellSum<T>) == sizeof(double), "a bin is 8 bytes");
+    unsigned int *const cnts = reinterpret_cast<unsigned int *>(shell_raw + size_t(warps) * nshell * sizeof(ShellSum<T>));
     for (int i = threadIdx.x; i < warps * nshell; i += blockDim.x) {
         sums[i].zero();
         cnts[i] = 0u;
@@ -485,7 +462,7 @@ __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict
             const int head = in ? 31 - __clz(int(heads & upto)) : lane;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
-                const ShellSum<T> o = v.up(d);
+                const ShellSum<T> o = shell_up(v, d);
                 if (lane - d >= head) v.add(o);
             }
             const bool tail = in && (lane == 31 || (((heads | ~on) >> (lane + 1)) & 1u));
@@ -827,17 +804,17 @@ cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs
 cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, const unsigned int *peak, double *S,
                           unsigned long long *cnt, cudaStream_t s)
 {
-    const int warps = shell_warps(nshell);
-    const uint64_t rows = uint64_t(b.ny / 2 + 1) * (b.nz / 2 + 1);
-    const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, 152 * 4));
-    const size_t sm = size_t(warps) * nshell * (sizeof(double) + sizeof(unsigned int));
-    if (prec == 0) {
-        cudaFuncSetAttribute(k_shells<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
-        k_shells<double><<<grid, 32 * warps, sm, s>>>(static_cast<const double *>(spec), b, nshell, peak, S, cnt);
-    } else {
-        cudaFuncSetAttribute(k_shells<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
-        k_shells<float><<<grid, 32 * warps, sm, s>>>(static_cast<const float *>(spec), b, nshell, peak, S, cnt);
-    }
+    auto run = [&](auto zero) {
+        using T = decltype(zero);
+        const int warps = shell_warps<T>(nshell);
+        const uint64_t rows = uint64_t(b.ny / 2 + 1) * (b.nz / 2 + 1);
+        const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, 152 * 4));
+        cudaFuncSetAttribute(k_shells<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
+        k_shells<T><<<grid, 32 * warps, warps * nshell * kShellBin<T>, s>>>(static_cast<const T *>(spec), b, nshell,
+                                                                            peak, S, cnt);
+    };
+    if (prec == 0) run(0.0);
+    else run(0.0f);
     return cudaGetLastError();
 }
 

@@ -54,6 +54,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "error_free.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 #include "normal_tab.cuh"
@@ -232,22 +233,6 @@ __device__ __forceinline__ R warp_sum(R v)
 constexpr int kFlushEvery = 8;
 
 template <typename R> struct TotSlot { R hi, lo; };
-
-// s + e = a + b exactly (round to nearest, no underflow).
-__device__ __forceinline__ float two_sum(float a, float b, float &e)
-{
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return s;
-}
-__device__ __forceinline__ double two_sum(double a, double b, double &e)
-{
-    const double s = __dadd_rn(a, b);
-    const double bb = __dsub_rn(s, a);
-    e = __dadd_rn(__dsub_rn(a, __dsub_rn(s, bb)), __dsub_rn(b, bb));
-    return s;
-}
 
 template <typename R>
 __device__ __forceinline__ void totals_init(TotSlot<R> (*tot)[NSTAT])
