@@ -224,10 +224,10 @@ __device__ __forceinline__ R warp_sum(R v)
 
 // Fused-reduction totals of a CTA, one slot per warp and sum (blockDim.x a
 // multiple of 32, at most 32 warps).  Threads add their nodes' terms in R;
-// every kFlushEvery rows (row pipeline) or chunks (direct kernel) each warp
-// adds its threads' partial sums (a warp_sum in R) to its slots and restarts
-// them, so that in FP32 no sum spans more than kFlushEvery rows of a
-// thread's nodes.  A slot is an unevaluated pair hi + lo kept by Knuth's
+// every kFlushEvery rows (k_step_rows) or kFlushEvery nodes of a thread (the
+// direct kernel, k_step_items) each warp adds its threads' partial sums (a
+// warp_sum in R) to its slots and restarts them, so that in FP32 no sum spans
+// more than the nodes of kFlushEvery rows, or 32 kFlushEvery = 256 nodes.  A slot is an unevaluated pair hi + lo kept by Knuth's
 // error-free TwoSum (no FP64 arithmetic in the loop: the FP64 pipe is slow),
 // and block_store_totals adds the slots in fixed warp order in FP64.
 constexpr int kFlushEvery = 8;
@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(kBlock, NP == 2 ? 3 : FLBM_MIN_BLOCKS) k_step(
     uint32_t it = 0;
     for (uint64_t base = n - threadIdx.x; base < a.n; base += stride, n += stride, ++it) {
         // CTA-uniform: every thread walks the same groups
-        if (STATS && it % kFlushEvery == kFlushEvery - 1) warp_flush(acc, tot);
+        if (STATS && it % (kFlushEvery / NP) == kFlushEvery / NP - 1) warp_flush(acc, tot);
         // a node past the end reads zeros (which add nothing to the sums) and
         // stores nothing
         const bool on = n < a.n, on2 = NP == 2 && n + kBlock < a.n;
@@ -1363,8 +1363,8 @@ __global__ void __launch_bounds__(kRowPairCompute + 32, row_pair_ctas<S>())
     k_step_items(S *__restrict__ g, const StepArgs<R> a, const RowItems items)
 {
     constexpr uint32_t nc = kRowPairCompute, stage_elems = uint32_t(kQ) * kItemNodes;
-    // a thread's nodes between two flushes: those of kFlushEvery 256-node rows
-    constexpr uint32_t kFlush = kFlushEvery * 256 / kItemNodes;
+    constexpr uint32_t kFlush = kFlushEvery * nc / kItemNodes;   // items of kFlushEvery nodes a thread
+    static_assert(kFlush * kItemNodes == kFlushEvery * nc, "whole items");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[2], empty[2];
     __shared__ TotSlot<R> tot[32][NSTAT];
