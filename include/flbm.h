@@ -89,7 +89,7 @@ enum flbm_status {
     FLBM_E_NOMEM = -2,       /* device or host allocation failed / buffer too small */
     FLBM_E_CUDA = -3,        /* a CUDA runtime / cuFFT call failed */
     FLBM_E_UNSTABLE = -4,    /* a step met rho <= 0 or a non-finite value */
-    FLBM_E_TIMEOUT = -5,     /* reserved: bounded device wait ran out */
+    FLBM_E_TIMEOUT = -5,     /* a bounded device wait ran out */
     FLBM_E_UNSUPPORTED = -6  /* valid request the library does not implement */
 };
 
@@ -452,7 +452,12 @@ int flbm_mlp_grad(const float *params, const float *dev_x, const float *dev_t, i
  * [0, n) drawn from seed), in mini-batches of `batch`; step size lr with a
  * cosine decay to 5 % over the run; beta1 0.9, beta2 0.999, eps 1e-8.
  * epoch_loss[epochs] (may be NULL) receives each epoch's mean loss over its
- * mini-batches (measured before each update). */
+ * mini-batches (measured before each update).
+ * Batches of up to 19,456 samples run as one cooperative launch per up to
+ * 1024 of them; where the process is not given every SM of the device, a
+ * launch per gradient, sum and update takes its place (sums in another
+ * order).  FLBM_E_TIMEOUT, with params unchanged, if a CTA waits seconds for
+ * the others (a bounded wait). */
 int flbm_mlp_train(float *params, const float *dev_x, const float *dev_t, int64_t n, int epochs, int batch,
                    double lr, uint64_t seed, double *epoch_loss);
 

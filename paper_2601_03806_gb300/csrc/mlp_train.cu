@@ -29,6 +29,7 @@
 // more kernels for the sums and Adam, took 130 us (8 of 152 SMs busy).
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <numeric>
 #include <random>
@@ -721,9 +722,11 @@ auto with_tile(int T, F &&f)
 
 constexpr uint64_t kTrainChunk = 1024;   // mini-batches of one training launch at most
 
-// A call's device workspace: one allocation, cut up by take().
+// A call's device workspace: one allocation, cut up by take(), and the partial
+// gradients of a training call whose cooperative launch was refused.
 struct Scratch {
     unsigned char *base = nullptr;
+    double *partials = nullptr;
     size_t used = 0;
     cudaStream_t s = nullptr;
     template <typename P>
@@ -736,6 +739,7 @@ struct Scratch {
     {
         if (s) cudaStreamSynchronize(s);
         cudaFree(base);
+        cudaFree(partials);
         if (s) cudaStreamDestroy(s);
     }
 };
@@ -827,6 +831,22 @@ int prepare(Scratch &sc, Work &w, const float *params, uint64_t B, uint64_t nb, 
     return FLBM_OK;
 }
 
+// Training continues without k_mlp_train: a gradient, its sums and Adam per
+// mini-batch, as for larger batches (three launches, slower, the same
+// accuracy: a partial sum spans a tile or two of samples).
+int without_cooperation(Scratch &sc, Work &w, uint64_t B)
+{
+    cudaGetLastError();   // clear the refusal
+    w.epochs_in_one = false;
+    w.grid = int(std::min<uint64_t>((B + w.T - 1) / w.T, uint64_t(2) * w.nsm));
+    const size_t bytes = (size_t(w.grid) * kNpPad + size_t(w.grid) * 8) * sizeof(double);
+    const cudaError_t e = cudaMalloc(&sc.partials, bytes);
+    if (e != cudaSuccess) return fail(std::string("mlp: cudaMalloc: ") + cudaGetErrorString(e), FLBM_E_NOMEM);
+    w.partials = sc.partials;
+    w.lpart = sc.partials + size_t(w.grid) * kNpPad;
+    return FLBM_OK;
+}
+
 float norm_of(uint64_t count) { return float(1.0 / (double(count) * kNout)); }
 
 // gradient (and loss sum) of batch b of the epoch order into w.grad
@@ -845,8 +865,17 @@ cudaError_t launch_grad(Scratch &sc, Work &w, const Samples &s, uint64_t b)
     return cudaGetLastError();
 }
 
+// Whether a cooperative launch was refused for want of the SMs or of the
+// feature: a process may hold only part of the device's SMs (MPS, green
+// contexts), and the grid takes every one that the device has.
+bool refused(cudaError_t e) { return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported; }
+
+// FLBM_INJECT_REFUSE=1 (environment, failure-injection tests only): the
+// cooperative launch is refused.
 cudaError_t launch_train(Scratch &sc, const Work &w, TrainArgs &a)
 {
+    const char *inject = std::getenv("FLBM_INJECT_REFUSE");
+    if (inject && std::atoi(inject) == 1) return cudaErrorCooperativeLaunchTooLarge;
     void *args[] = {&a};
     return with_tile(w.T, [&](auto tag) {
         constexpr int T = decltype(tag)::value;
@@ -926,29 +955,35 @@ extern "C" int flbm_mlp_train(float *params, const float *dev_x, const float *de
             off = rng() % N;
         }
         const Samples s{dev_x, dev_t, N, B, mult, off};
+        uint64_t b = 0, planned = 0;   // the next batch; step sizes drawn so far
         if (w.epochs_in_one) {
-            for (uint64_t b = 0; b < nb && e == cudaSuccess; b += kTrainChunk) {
+            for (; b < nb && e == cudaSuccess; b = planned) {
                 const uint64_t b1 = std::min(b + kTrainChunk, nb);
                 for (uint64_t k = b; k < b1; ++k) lrs[k] = next_lr();
+                planned = b1;
                 TrainArgs a{s,     b,     b1,   norm_of(B), norm_of(N - (nb - 1) * B), beta1,  beta2, eps, w.img, w.m1,
                             w.m2,  w.lr,  w.act, w.stride, w.lpart, w.loss, w.bar, w.bar + 1};
                 e = cudaMemcpyAsync(w.lr, lrs.data() + b, (b1 - b) * sizeof(float), cudaMemcpyHostToDevice, sc.s);
                 if (e == cudaSuccess) e = cudaMemsetAsync(w.bar, 0, sizeof(unsigned int), sc.s);
                 if (e == cudaSuccess) e = launch_train(sc, w, a);
+                if (refused(e)) {
+                    if ((rc = without_cooperation(sc, w, B)) != FLBM_OK) return rc;
+                    e = cudaSuccess;
+                    break;
+                }
             }
-        } else {
-            for (uint64_t b = 0; b < nb && e == cudaSuccess; ++b) {
-                e = launch_grad(sc, w, s, b);
-                if (e != cudaSuccess) break;
-                e = cudaMemcpyAsync(w.loss + b, w.grad + kNp, sizeof(double), cudaMemcpyDeviceToDevice, sc.s);
-                k_mlp_adam<<<(kNp + 255) / 256, 256, 0, sc.s>>>(w.img, w.m1, w.m2, w.grad, next_lr(), beta1, beta2,
-                                                                eps);
-                if (e == cudaSuccess) e = cudaGetLastError();
-            }
+        }
+        for (; b < nb && e == cudaSuccess; ++b) {
+            e = launch_grad(sc, w, s, b);
+            if (e != cudaSuccess) break;
+            e = cudaMemcpyAsync(w.loss + b, w.grad + kNp, sizeof(double), cudaMemcpyDeviceToDevice, sc.s);
+            const float lr_b = b < planned ? lrs[b] : next_lr();
+            k_mlp_adam<<<(kNp + 255) / 256, 256, 0, sc.s>>>(w.img, w.m1, w.m2, w.grad, lr_b, beta1, beta2, eps);
+            if (e == cudaSuccess) e = cudaGetLastError();
         }
         if (e != cudaSuccess) break;
         e = cudaMemcpyAsync(h.data(), w.loss, sizeof(double) * nb, cudaMemcpyDeviceToHost, sc.s);
-        if (e == cudaSuccess && w.epochs_in_one)
+        if (e == cudaSuccess && w.bar)
             e = cudaMemcpyAsync(book, w.bar, sizeof(book), cudaMemcpyDeviceToHost, sc.s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(sc.s);
         if (e == cudaSuccess && (book[1] & 2u))
