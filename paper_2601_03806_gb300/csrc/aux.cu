@@ -94,7 +94,7 @@ __global__ void k_fill_zero(S *g, uint64_t count)
 
 // out[i*cn + k] = f_i (absolute, or deviation) at node n0 + k
 template <typename S>
-__global__ void k_gather_f(const S *g, BoxDesc b, uint64_t n0, uint64_t cn, double *out, int dev)
+__global__ void k_gather_f(const S *g, BoxDesc b, uint64_t n0, uint64_t cn, double *out)
 {
     for (uint64_t k = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; k < cn;
          k += uint64_t(gridDim.x) * blockDim.x) {
@@ -109,7 +109,7 @@ __global__ void k_gather_f(const S *g, BoxDesc b, uint64_t n0, uint64_t cn, doub
                     const int i = slot_of(cx, cy, cz);
                     const double w = w1(cx) * w1(cy) * w1(cz);
                     const double gv = ldd(g, storage_index(cx, cy, cz, x, y, z, b));
-                    out[uint64_t(i) * cn + k] = dev ? gv : gv + w * b.rho0;
+                    out[uint64_t(i) * cn + k] = gv + w * b.rho0;
                 }
     }
 }
@@ -682,12 +682,12 @@ cudaError_t launch_fill_rest(void *g, int prec, uint64_t count, cudaStream_t s)
 }
 
 cudaError_t launch_gather_f(const void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,
-                            double *out, bool deviations, cudaStream_t s)
+                            double *out, cudaStream_t s)
 {
     const int grid = grid_for(cn, 128);
     with_storage(prec, [&](auto tag) {
         using S = decltype(tag);
-        k_gather_f<S><<<grid, 128, 0, s>>>(static_cast<const S *>(g), b, n0, cn, out, deviations);
+        k_gather_f<S><<<grid, 128, 0, s>>>(static_cast<const S *>(g), b, n0, cn, out);
     });
     return cudaGetLastError();
 }

@@ -760,7 +760,7 @@ int flbm_get_populations(flbm_ctx *c, double *f)
     const int prec = prec_code(c);
     return d2h_chunks(
         c, [&](double *buf, uint64_t n0, uint64_t cn) {
-            return launch_gather_f(c->g, prec, b, n0, cn, buf, false, c->stream);
+            return launch_gather_f(c->g, prec, b, n0, cn, buf, c->stream);
         },
         [&](double *buf, uint64_t n0, uint64_t cn) {
             const size_t w = cn * sizeof(double);

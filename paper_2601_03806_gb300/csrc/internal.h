@@ -253,7 +253,7 @@ struct BoxDesc {
 };
 cudaError_t launch_fill_rest(void *g, int prec, uint64_t count, cudaStream_t s);
 cudaError_t launch_gather_f(const void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,
-                            double *out, bool deviations, cudaStream_t s);
+                            double *out, cudaStream_t s);
 cudaError_t launch_gather_state(const void *g, int prec, const BoxDesc &b, uint64_t n0,
                                 uint64_t cn, void *out, cudaStream_t s);
 cudaError_t launch_scatter_f(void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,
