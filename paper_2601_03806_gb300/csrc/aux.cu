@@ -794,7 +794,7 @@ cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs
         // aligned buffer) starting on 16 bytes
         const bool vec = b.parity == 0 && b.n % V == 0 && b.ns % V == 0;
         const uint64_t groups = vec ? b.n / V : b.n;
-        const int grid = int(std::min<uint64_t>((groups + 255) / 256, 152 * 16));
+        const int grid = int(std::min<uint64_t>((groups + 255) / 256, uint64_t(b.nsm) * 16));
         if (vec) observable<S, V>(g, b, obs, field, peak, grid, s);
         else observable<S, 1>(g, b, obs, field, peak, grid, s);
     });
@@ -808,7 +808,7 @@ cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshe
         using T = decltype(zero);
         const int warps = shell_warps<T>(nshell);
         const uint64_t rows = uint64_t(b.ny / 2 + 1) * (b.nz / 2 + 1);
-        const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, 152 * 4));
+        const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, uint64_t(b.nsm) * 4));
         cudaFuncSetAttribute(k_shells<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
         k_shells<T><<<grid, 32 * warps, warps * nshell * kShellBin<T>, s>>>(static_cast<const T *>(spec), b, nshell,
                                                                             peak, S, cnt);

@@ -114,6 +114,7 @@ BoxDesc box_of(const flbm_ctx *c)
     b.ns = c->ns;
     b.rho0 = c->p.rho0;
     b.parity = parity(c);
+    b.nsm = c->nsm;
     return b;
 }
 
@@ -213,6 +214,7 @@ StepArgs<R> make_args(const flbm_ctx *c, int64_t t, double *partials = nullptr, 
     fill_constants_t<R>(c->p, a);
     a.tx_pad = c->tx_pad;
     a.normals = c->normals;
+    a.nsm = uint32_t(c->nsm);
     a.chained = chained;
     a.partials = partials;
     a.flag = &c->dflags->flag;
@@ -398,7 +400,9 @@ int flbm::create_ctx(const flbm_params *p, void *dev_buf, size_t dev_bytes, void
     const auto step_shape = p->precision == FLBM_FP64   ? step_shape_f64
                             : p->precision == FLBM_FP32 ? step_shape_f32
                                                         : step_shape_f16;
-    step_grids(*p, c->nsm, step_shape(p->scheme, uint32_t(p->nx), uint32_t(p->ny), uint32_t(p->nz), c->ns, true), c->grid, c->row_grid);
+    step_grids(*p, c->nsm,
+               step_shape(p->scheme, uint32_t(p->nx), uint32_t(p->ny), uint32_t(p->nz), c->ns, true, c->nsm), c->grid,
+               c->row_grid);
     // FLBM_INJECT_STARVE=1 (environment, failure-injection tests only): the
     // row pipeline expects 16 bytes more than it copies (the learned step
     // issues no first-layer MMA), so the bounded waits run out and flbm_step

@@ -45,6 +45,7 @@ struct StepArgs {
     int32_t noise_rho0;           // phi_k uses rho0 instead of rho(x,t)
     uint32_t tx_pad;              // failure injection: bytes the row pipeline
                                   // expects beyond what it copies (0 normally)
+    uint32_t nsm;                 // host: SMs of the device
     uint32_t chained;             // host: the stream's last work is a step kernel or the totals of
                                   // steps, and this launch may overlap its end (launch_step)
     R rho0;
@@ -158,9 +159,9 @@ cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool 
 // Nodes from which the direct kernel takes two per thread in CTAs of kBlock
 // threads (below, one per thread in CTAs of a warp).
 constexpr uint64_t kDirectPairs = 65536;
-// FP64 nodes up to which an SM's warps share 32 of them (k_step_few; 152 SMs);
+// FP64 nodes per SM up to which an SM's warps share 32 of them (k_step_few);
 // larger boxes keep the FP64 units busy with a warp per 32 nodes.
-constexpr uint64_t kDirectFew = 4864;
+constexpr uint64_t kDirectFew = 32;
 // Launch shape of the step kernels for a box: the direct kernel's CTAs and how many of them an SM holds, and the row
 // pipeline's CTAs per SM (0 when it does not serve rows of length nx); the
 // slab stride ns picks the index width.  Also prepares the kernels'
@@ -169,9 +170,9 @@ struct StepShape {
     uint64_t ctas = 1, work = 0;   // of the direct kernel; work items of the row pipeline
     int direct = 1, rows = 0;
 };
-StepShape step_shape_f64(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
-StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
-StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats);
+StepShape step_shape_f64(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm);
+StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm);
+StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm);
 // Nodes from which boxes whose rows the pipeline can take run it (FP32 / FP16,
 // FP64); smaller ones run the direct kernel, which needs no fill and drain.
 constexpr uint64_t kRowsFrom = uint64_t(1) << 19, kRowsFrom64 = uint64_t(1) << 16;
@@ -250,6 +251,7 @@ struct BoxDesc {
     uint64_t ns;           // slab stride of the population storage (>= n)
     double rho0;
     int parity;            // 0: storage natural; 1: AA-shifted (odd form)
+    int nsm;               // SMs of the device
 };
 cudaError_t launch_fill_rest(void *g, int prec, uint64_t count, cudaStream_t s);
 cudaError_t launch_gather_f(const void *g, int prec, const BoxDesc &b, uint64_t n0, uint64_t cn,

@@ -112,7 +112,9 @@ extern "C" int flbm_step_noalloc(const flbm_params *p, void *dev_state, int64_t 
     const uint64_t n = uint64_t(p->nx) * uint64_t(p->ny) * uint64_t(p->nz);
     const uint64_t nchunks = uint64_t((p->nx + kBlock - 1) / kBlock) * p->ny * p->nz;
     int grid = 0, row_grid = 0;
-    step_grids(*p, nsm, step_shape_f32(p->scheme, uint32_t(p->nx), uint32_t(p->ny), uint32_t(p->nz), n, true), grid, row_grid);
+    step_grids(*p, nsm,
+               step_shape_f32(p->scheme, uint32_t(p->nx), uint32_t(p->ny), uint32_t(p->nz), n, true, nsm), grid,
+               row_grid);
     const int used = row_grid > 0 ? row_grid : grid;
     if (used > kNoallocMaxCtas)
         return noalloc_fail(FLBM_E_INVALID,
@@ -128,6 +130,7 @@ extern "C" int flbm_step_noalloc(const flbm_params *p, void *dev_state, int64_t 
     a.n = n;
     a.ns = n;   // the caller's state: 27 unpadded slabs
     a.nchunks = nchunks;
+    a.nsm = uint32_t(nsm);
     a.step = uint64_t(step);
     fill_step_constants(*p, a);
     a.partials = sc->partials;

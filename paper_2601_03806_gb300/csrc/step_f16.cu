@@ -23,10 +23,10 @@ cudaError_t launch_step_f16(void *g, const StepArgs<float> &a, int scheme, bool 
     return launch_step_t<__half, float, uint64_t>(h, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats)
+StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm)
 {
-    StepShape s = fits32(ns) ? step_shape_t<__half, float, uint32_t>(scheme, nx, ny, nz, stats)
-                             : step_shape_t<__half, float, uint64_t>(scheme, nx, ny, nz, stats);
+    StepShape s = fits32(ns) ? step_shape_t<__half, float, uint32_t>(scheme, nx, ny, nz, stats, nsm)
+                             : step_shape_t<__half, float, uint64_t>(scheme, nx, ny, nz, stats, nsm);
     const RowPlan rp = row_plan<__half>(nx, ny, nz);
     if (rp.grouped) {
         s.rows = items_resident_f16(scheme, nx, ny, nz);

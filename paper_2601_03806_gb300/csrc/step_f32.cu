@@ -21,10 +21,10 @@ cudaError_t launch_step_f32(float *g, const StepArgs<float> &a, int scheme, bool
     return launch_step_t<float, float, uint64_t>(g, a, scheme, odd, stats, grid, row_grid, s);
 }
 
-StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats)
+StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm)
 {
-    StepShape s = fits32(ns) ? step_shape_t<float, float, uint32_t>(scheme, nx, ny, nz, stats)
-                             : step_shape_t<float, float, uint64_t>(scheme, nx, ny, nz, stats);
+    StepShape s = fits32(ns) ? step_shape_t<float, float, uint32_t>(scheme, nx, ny, nz, stats, nsm)
+                             : step_shape_t<float, float, uint64_t>(scheme, nx, ny, nz, stats, nsm);
     const RowPlan rp = row_plan<float>(nx, ny, nz);
     if (rp.grouped) {
         s.rows = items_resident_f32(scheme, nx, ny, nz);

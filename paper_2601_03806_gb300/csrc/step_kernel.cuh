@@ -1645,12 +1645,12 @@ struct DirectPlan {
     bool few = false;   // k_step_few (FP64)
 };
 template <typename S>
-inline DirectPlan direct_plan(uint64_t n)
+inline DirectPlan direct_plan(uint64_t n, uint32_t nsm)
 {
     DirectPlan p;
     p.np = !std::is_same<S, double>::value && row_pairs_enabled() && n >= kDirectPairs ? 2 : 1;
     p.threads = n >= kDirectPairs ? kBlock : 32;
-    p.few = std::is_same<S, double>::value && n <= kDirectFew;
+    p.few = std::is_same<S, double>::value && n <= kDirectFew * nsm;
     const uint64_t span = uint64_t(p.np) * p.threads;
     p.ctas = (n + span - 1) / span;
     return p;
@@ -1676,7 +1676,7 @@ cudaError_t launch_step_t(S *g, const StepArgs<R> &a, int scheme, bool odd, bool
 #undef FLBM_LAUNCH_ROWS
         return cudaGetLastError();
     }
-    const DirectPlan dp = direct_plan<S>(a.n);
+    const DirectPlan dp = direct_plan<S>(a.n, a.nsm);
 #define FLBM_LAUNCH(SC, OD, ST) launch_direct<S, R, I, SC, OD, ST>(g, a, dp, grid, s)
     if (scheme == 0) {
         if (odd) { if (stats) FLBM_LAUNCH(0, true, true); else FLBM_LAUNCH(0, true, false); }
@@ -1777,9 +1777,9 @@ int direct_resident(const DirectPlan &dp, bool stats)
 // row pipeline does not serve the box); also opts the row kernels into their
 // shared memory on the current device.
 template <typename S, typename R, typename I, int SC>
-void prepare_scheme(uint32_t nx, uint32_t ny, uint32_t nz, bool stats, StepShape &shape)
+void prepare_scheme(uint32_t nx, uint32_t ny, uint32_t nz, bool stats, int nsm, StepShape &shape)
 {
-    const DirectPlan dp = direct_plan<S>(uint64_t(nx) * ny * nz);
+    const DirectPlan dp = direct_plan<S>(uint64_t(nx) * ny * nz, uint32_t(nsm));
     shape.ctas = dp.ctas;
     shape.rows = 0;
     if constexpr (std::is_same<S, double>::value) {
@@ -1805,12 +1805,12 @@ void prepare_scheme(uint32_t nx, uint32_t ny, uint32_t nz, bool stats, StepShape
 }
 
 template <typename S, typename R, typename I>
-StepShape step_shape_t(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, bool stats)
+StepShape step_shape_t(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, bool stats, int nsm)
 {
     StepShape shape;
-    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, ny, nz, stats, shape);
-    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, ny, nz, stats, shape);
-    else prepare_scheme<S, R, I, 2>(nx, ny, nz, stats, shape);
+    if (scheme == 0) prepare_scheme<S, R, I, 0>(nx, ny, nz, stats, nsm, shape);
+    else if (scheme == 1) prepare_scheme<S, R, I, 1>(nx, ny, nz, stats, nsm, shape);
+    else prepare_scheme<S, R, I, 2>(nx, ny, nz, stats, nsm, shape);
     return shape;
 }
 
