@@ -463,12 +463,13 @@ void step_grids(const flbm_params &p, int nsm, const StepShape &shape, int &grid
     grid = int(std::min<uint64_t>(work, uint64_t(nsm) * per_sm));
     if (grid < 1) grid = 1;
     // FLBM_ROWS (environment): 0 disables the TMA row pipeline, 1 runs it for
-    // small boxes too, as failure injection does (its waits are what runs out)
+    // small and thin boxes too, as failure injection does (its waits are what
+    // runs out)
     row_grid = 0;
     const char *rows_env = std::getenv("FLBM_ROWS"), *inject = std::getenv("FLBM_INJECT_STARVE");
     const int rows = rows_env ? std::atoi(rows_env) : (inject && std::atoi(inject) == 1 ? 1 : -1);
-    const bool small = n < (p.precision == FLBM_FP64 ? kRowsFrom64 : kRowsFrom);
-    if (shape.rows > 0 && p.scheme != FLBM_LEARNED && rows != 0 && (rows == 1 || !small)) {
+    const bool fits = n >= (p.precision == FLBM_FP64 ? kRowsFrom64 : kRowsFrom) && shape.item >= kItemLeast;
+    if (shape.rows > 0 && p.scheme != FLBM_LEARNED && rows != 0 && (rows == 1 || fits)) {
         row_grid = int(std::min<uint64_t>(shape.work, uint64_t(nsm) * shape.rows));
     }
 }

@@ -162,13 +162,14 @@ constexpr uint64_t kDirectPairs = 65536;
 // FP64 nodes per SM up to which an SM's warps share 32 of them (k_step_few);
 // larger boxes keep the FP64 units busy with a warp per 32 nodes.
 constexpr uint64_t kDirectFew = 32;
-// Launch shape of the step kernels for a box: the direct kernel's CTAs and how many of them an SM holds, and the row
-// pipeline's CTAs per SM (0 when it does not serve rows of length nx); the
-// slab stride ns picks the index width.  Also prepares the kernels'
-// shared-memory attributes on the current device.
+// Launch shape of the step kernels for a box: the direct kernel's CTAs and how
+// many of them an SM holds, and the row pipeline's CTAs per SM (0 when it does
+// not serve rows of length nx); the slab stride ns picks the index width.
+// Also prepares the kernels' shared-memory attributes on the current device.
 struct StepShape {
     uint64_t ctas = 1, work = 0;   // of the direct kernel; work items of the row pipeline
     int direct = 1, rows = 0;
+    uint32_t item = ~0u;           // nodes of a work item of grouped rows
 };
 StepShape step_shape_f64(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm);
 StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint64_t ns, bool stats, int nsm);
@@ -176,6 +177,13 @@ StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint
 // Nodes from which boxes whose rows the pipeline can take run it (FP32 / FP16,
 // FP64); smaller ones run the direct kernel, which needs no fill and drain.
 constexpr uint64_t kRowsFrom = uint64_t(1) << 19, kRowsFrom64 = uint64_t(1) << 16;
+// Nodes of a work item of grouped rows from which the pipeline is the default.
+// An item takes the rows of one plane, and its waits cost the same whatever it
+// holds, so boxes of short rows and few of them a plane leave most of a CTA
+// idle: 32 x 1 x 65,536 FP32 541 us a step, 95 on the direct kernel; items of
+// 192 nodes (96 x 2 x 16,384) 195 and 142; of 224 (224 x 1 x 8,192) 91 and 85,
+// FP16 74 and 78; of 256 (64 x 4 x 8,192) 103 and 93, FP16 82 and 88.
+constexpr uint32_t kItemLeast = 224;
 // The grouped-row kernels (step_f32_items.cu, step_f16_items.cu) of boxes
 // whose row_plan is grouped.
 cudaError_t launch_items_f32(float *g, const StepArgs<float> &a, int scheme, bool odd, bool stats, int row_grid,

@@ -31,6 +31,7 @@ StepShape step_shape_f16(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint
     if (rp.grouped) {
         s.rows = items_resident_f16(scheme, nx, ny, nz);
         s.work = rp.work;
+        s.item = rp.item.rows * nx;
     } else if (s.rows > 0 && rows_fixed<512>(rp, nx)) {
         s.rows = rows_occupancy_f16_nx512(scheme, stats, ny, nz);
     }

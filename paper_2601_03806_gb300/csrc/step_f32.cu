@@ -29,6 +29,7 @@ StepShape step_shape_f32(int scheme, uint32_t nx, uint32_t ny, uint32_t nz, uint
     if (rp.grouped) {
         s.rows = items_resident_f32(scheme, nx, ny, nz);
         s.work = rp.work;
+        s.item = rp.item.rows * nx;
     } else if (rows_paced<float>(rp)) {
         s.rows = rows_occupancy_f32_paced(scheme, stats, nx, ny, nz);
     }

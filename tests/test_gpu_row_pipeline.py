@@ -113,6 +113,29 @@ def test_the_named_kernel_runs(F, prec, shape, name):
     box.close()
 
 
+# boxes of 2^19 nodes and more: grouped rows from 224 nodes an item
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+@pytest.mark.parametrize("shape,name", [((32, 1, 16384), "k_step<"), ((32, 6, 2731), "k_step<"),
+                                        ((64, 3, 2731), "k_step<"), ((96, 2, 2731), "k_step<"),
+                                        ((32, 7, 2341), "k_step_items"), ((64, 4, 2048), "k_step_items"),
+                                        ((224, 1, 2341), "k_step_items"), ((256, 1, 2048), "k_step_items")])
+def test_thin_boxes_take_the_direct_kernel(F, monkeypatch, prec, shape, name):
+    """By default, and with the same populations as the pipeline's."""
+    a = F.Lattice(*shape, 0.7, 1e-4, seed=3, precision=prec)
+    monkeypatch.delenv("FLBM_ROWS")
+    b = F.Lattice(*shape, 0.7, 1e-4, seed=3, precision=prec)
+    for box in (a, b):
+        box.init_thermal(6)
+        box.step(1)
+    got = kernels(lambda: b.step(2))
+    assert any(name in k for k in got), got
+    assert not any("k_step" in k and name not in k for k in got), got
+    a.step(b.step_count - a.step_count)
+    assert np.array_equal(a.get_state(), b.get_state())
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("shape", [(64, 6, 5), (96, 5, 3), (256, 3, 2), (288, 3, 2), (512, 3, 2)])
 def test_the_call_without_allocation_matches(F, oracle_mod, shape):
     import torch
