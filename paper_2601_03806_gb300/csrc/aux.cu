@@ -1,7 +1,7 @@
 // aux.cu -- non-hot kernels: initial state, AA-aware gather/scatter of the
 // populations, moment export (Eqs. rho/u and Pi), observable fields and the
-// FP64 shell binning of S(k) (Sec. III), and the final pass of the fused
-// reductions.
+// shell binning of S(k) (Sec. III; sums as good as FP64's, FP64 totals), and
+// the final pass of the fused reductions.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -355,18 +355,19 @@ __device__ __forceinline__ ShellSum<double> shell_up(const ShellSum<double> &v, 
     return ShellSum<double>{__shfl_up_sync(0xffffffffu, v.v, d)};
 }
 
-// Power of two that brings a spectrum whose field peaks at `peak` into a
-// range where FP32 squares neither overflow nor underflow: every amplitude is
-// at most N peak, and so is the root of the sum of all squares (Parseval);
-// N peak goes to about 2^60.  Exact, and divided out of the totals.
-__device__ __forceinline__ float shell_scale(unsigned int peak_bits, uint64_t n)
+// k of the power of two 2^k that brings a spectrum whose field peaks at `peak`
+// (its bits) into a range where FP32 squares neither overflow nor underflow:
+// every amplitude is at most N peak, and so is the root of the sum of all
+// squares (Parseval); N peak goes to about 2^60.  Exact, and divided out of
+// the totals.
+__device__ __forceinline__ int shell_scale(unsigned int peak, uint64_t n)
 {
-    const float peak = __uint_as_float(peak_bits);
-    if (!(peak > 0.0f) || !(peak < INFINITY)) return 1.0f;
-    int k = 60 - (ilogb(double(peak)) + 1) - (64 - __clzll((long long)n));
-    k = k > 126 ? 126 : (k < -126 ? -126 : k);
-    return __uint_as_float(uint32_t(127 + k) << 23);
+    if (peak == 0u || peak >= 0x7f800000u) return 0;
+    const int k = 60 - (int(peak >> 23) - 127 + 1) - (64 - __clzll((long long)n));
+    return k > 126 ? 126 : (k < -126 ? -126 : k);
 }
+__device__ __forceinline__ float power2(int k, float) { return __uint_as_float(uint32_t(127 + k) << 23); }
+__device__ __forceinline__ double power2(int k, double) { return __longlong_as_double((long long)(1023 + k) << 52); }
 
 // round(|n|) of n2 = |n|^2: 0, or the s >= 1 with s^2 - s < n2 <= s^2 + s (|n|
 // is never a half-integer), from a square root good to one.
@@ -376,6 +377,16 @@ __device__ __forceinline__ long long shell_of(unsigned long long n2)
     long long s = n2 < (1ull << 44) ? (long long)(__fsqrt_rn(float(n2)) + 0.5f) : llrint(sqrt(double(n2)));
     while (s * s - s >= (long long)n2) --s;
     while (s * s + s < (long long)n2) ++s;
+    return s;
+}
+
+// The same for n2 < 2^31, in 32 bits.
+__device__ __forceinline__ uint32_t shell_of(uint32_t n2)
+{
+    if (n2 == 0) return 0;
+    uint32_t s = uint32_t(__fsqrt_rn(float(n2)) + 0.5f);
+    while (s * s - s >= n2) --s;
+    while (s * s + s < n2) ++s;
     return s;
 }
 
@@ -391,16 +402,42 @@ int shell_warps(int nshell)
     return w < size_t(kShellWarps) ? int(w) : kShellWarps;
 }
 
+// The lane's sum of the squares of up to four complex elements.
+__device__ __forceinline__ ShellSum<float> square_sum(const float (&re)[4], const float (&im)[4])
+{
+    TripleSum<float2> w;   // real and imaginary parts, a lane each
+    w.hi = w.mid = w.lo = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w.add_square(make_float2(re[q], im[q]));
+    ShellSum<float> v;
+    v.hi = w.hi.x;
+    v.mid = w.mid.x;
+    v.lo = w.lo.x + w.lo.y;
+    v.add(w.hi.y, w.mid.y);
+    return v;
+}
+__device__ __forceinline__ ShellSum<double> square_sum(const double (&re)[4], const double (&im)[4])
+{
+    ShellSum<double> v;
+    v.zero();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        v.add_square(re[q]);
+        v.add_square(im[q]);
+    }
+    return v;
+}
+
 // A warp takes the rows kx = 0 .. nx/2 of (+-ky, +-kz), up to four at once:
 // they have the same |n| element by element, so one shell index and one
 // binning serve four values.  Along a row the shell only grows, so lanes of
-// one shell are neighbours: a segmented scan leaves each shell's sum on its
-// last lane, which adds it to the warp's own bins in shared memory -- no
-// atomics until the CTA's totals, added in FP64.  Rows stop at the last
-// shell asked for.
+// one shell are neighbours: a segmented scan, as deep as the longest segment
+// needs, leaves each shell's sum on its last lane, which adds it to the warp's
+// own bins in shared memory -- no atomics until the CTA's totals, added in
+// FP64.  Rows stop at the last shell asked for.
 template <typename T>
 __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict__ spec, const BoxDesc b, int nshell,
-                                                             const unsigned int *peak, double *S,
+                                                             double inv_n, const unsigned int *peak, double *S,
                                                              unsigned long long *cnt)
 {
     extern __shared__ __align__(16) unsigned char shell_raw[];
@@ -412,24 +449,40 @@ __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict
         cnts[i] = 0u;
     }
     __syncthreads();
+    using C = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
+    const C *const elems = reinterpret_cast<const C *>(spec);
     ShellSum<T> *const bin = sums + size_t(warp) * nshell;
     unsigned int *const num = cnts + size_t(warp) * nshell;
     const uint32_t nxh = b.nx / 2 + 1, nyh = b.ny / 2 + 1, nzh = b.nz / 2 + 1;
-    const float scale = std::is_same<T, float>::value ? shell_scale(*peak, b.n) : 1.0f;
-    const uint64_t rows = uint64_t(nyh) * nzh;
-    for (uint64_t r = blockIdx.x * uint64_t(warps) + warp; r < rows; r += uint64_t(gridDim.x) * warps) {
-        const uint32_t ay = uint32_t(r % nyh), az = uint32_t(r / nyh);
+    auto square = [](uint64_t v) { return v * v; };
+    // every |n|^2, of the lanes past a row's end too, is below 2^31
+    const bool narrow = square(nxh + 31) + square(nyh) + square(nzh) < (uint64_t(1) << 31);
+    const int k2 = std::is_same<T, float>::value ? shell_scale(*peak, b.n) : 0;
+    const T scale = power2(k2, T(0));
+    // rows r = warp's index, + warps in all, ...: (ay, az) = (r % nyh, r / nyh), stepped without a division
+    const uint32_t first = blockIdx.x * uint32_t(warps) + warp, step = gridDim.x * uint32_t(warps);
+    uint32_t ay = first % nyh, az = first / nyh;
+    auto next = [&] {
+        ay += step % nyh;
+        az += step / nyh;
+        if (ay >= nyh) {
+            ay -= nyh;
+            ++az;
+        }
+    };
+    for (; az < nzh; next()) {
         const bool two_y = ay != 0 && 2 * uint64_t(ay) != b.ny, two_z = az != 0 && 2 * uint64_t(az) != b.nz;
         const unsigned long long perp = (unsigned long long)ay * ay + (unsigned long long)az * az;
         const int mult = (two_y ? 2 : 1) * (two_z ? 2 : 1);
-        const T *row[4];   // (ky, kz), (-ky, kz), (ky, -kz), (-ky, -kz)
-        row[0] = spec + 2 * (uint64_t(az) * b.ny + ay) * nxh;
-        row[1] = spec + 2 * (uint64_t(az) * b.ny + (b.ny - ay)) * nxh;
-        row[2] = spec + 2 * (uint64_t(b.nz - az) * b.ny + ay) * nxh;
-        row[3] = spec + 2 * (uint64_t(b.nz - az) * b.ny + (b.ny - ay)) * nxh;
+        const C *row[4];   // (ky, kz), (-ky, kz), (ky, -kz), (-ky, -kz)
+        row[0] = elems + (uint64_t(az) * b.ny + ay) * nxh;
+        row[1] = elems + (uint64_t(az) * b.ny + (b.ny - ay)) * nxh;
+        row[2] = elems + (uint64_t(b.nz - az) * b.ny + ay) * nxh;
+        row[3] = elems + (uint64_t(b.nz - az) * b.ny + (b.ny - ay)) * nxh;
         for (uint32_t k0 = 0; k0 < nxh; k0 += 32) {
             const uint32_t kx = k0 + lane;
-            const long long s = shell_of((unsigned long long)kx * kx + perp);
+            const long long s = narrow ? (long long)shell_of(kx * kx + uint32_t(perp))
+                                       : shell_of((unsigned long long)kx * kx + perp);
             const bool in = kx < nxh && s < nshell;
             // lanes of one row: in holds on a prefix of the warp
             const unsigned int on = __ballot_sync(0xffffffffu, in);
@@ -437,33 +490,28 @@ __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict
             // the conjugate half (kx -> -kx) has the same |n|; kx = 0 and the
             // even Nyquist plane are their own partners
             const bool own = kx == 0 || (b.nx % 2 == 0 && kx == b.nx / 2);
-            ShellSum<T> v;
-            v.zero();
-            if (in) {
-                T re[4], im[4];
+            T re[4], im[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const bool use = (!(q & 1) || two_y) && (!(q & 2) || two_z);
-                    re[q] = use ? row[q][2 * kx] * T(scale) : T(0);
-                    im[q] = use ? row[q][2 * kx + 1] * T(scale) : T(0);
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    v.add_square(re[q]);
-                    v.add_square(im[q]);
-                }
-                if (!own) v.scale2();
+            for (int q = 0; q < 4; ++q) {
+                const bool use = in && (!(q & 1) || two_y) && (!(q & 2) || two_z);
+                const C f = use ? row[q][kx] : C{};
+                re[q] = f.x * scale;
+                im[q] = f.y * scale;
             }
+            ShellSum<T> v = square_sum(re, im);
+            if (!own) v.scale2();
             const int sh = in ? int(s) : -1;
             const int left = __shfl_up_sync(0xffffffffu, sh, 1);
             const unsigned int heads = __ballot_sync(0xffffffffu, in && (lane == 0 || left != sh));
             const unsigned int owns = __ballot_sync(0xffffffffu, in && own);
             const unsigned int upto = 0xffffffffu >> (31 - lane);        // lanes 0 .. lane
             const int head = in ? 31 - __clz(int(heads & upto)) : lane;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
+            // bit l of runs: lanes l - d .. l are of one shell
+            unsigned int runs = on & ~heads;
+            for (int d = 1; runs; d <<= 1) {
                 const ShellSum<T> o = shell_up(v, d);
                 if (lane - d >= head) v.add(o);
+                runs &= runs << d;
             }
             const bool tail = in && (lane == 31 || (((heads | ~on) >> (lane + 1)) & 1u));
             if (tail && sh > 0) {   // shell 0 holds only n = 0, which is excluded
@@ -475,19 +523,67 @@ __global__ void __launch_bounds__(32 * kShellWarps) k_shells(const T *__restrict
         }
     }
     __syncthreads();
-    const double inv = 1.0 / (double(b.n) * double(scale) * double(scale));
+    const double inv = inv_n * power2(-2 * k2, 0.0);
     for (int s = threadIdx.x; s < nshell; s += blockDim.x) {
         double t = 0.0;
         unsigned long long k = 0;
         for (int w = 0; w < warps; ++w) {
+            const unsigned int c = cnts[size_t(w) * nshell + s];
+            if (!c) continue;   // most, where a warp takes a row or two
             t += sums[size_t(w) * nshell + s].value();
-            k += cnts[size_t(w) * nshell + s];
+            k += c;
         }
         if (k) {
             atomicAdd(&S[s], t * inv);
             atomicAdd(&cnt[s], k);
         }
     }
+}
+
+// The same sums element by element, in FP64, into the CTA's bins in shared
+// memory by atomics: for spectra whose rows are too few, or too short, to fill
+// the warps of k_shells (shells_flat).
+template <typename T>
+__global__ void __launch_bounds__(256) k_shells_flat(const T *__restrict__ spec, const BoxDesc b, int nshell,
+                                                     double inv_n, double *S, unsigned long long *cnt)
+{
+    extern __shared__ __align__(16) unsigned char shell_raw[];
+    double *const sums = reinterpret_cast<double *>(shell_raw);
+    unsigned long long *const cnts = reinterpret_cast<unsigned long long *>(sums + nshell);
+    for (int s = threadIdx.x; s < nshell; s += blockDim.x) {
+        sums[s] = 0.0;
+        cnts[s] = 0ull;
+    }
+    __syncthreads();
+    const uint32_t nxh = b.nx / 2 + 1;
+    const uint64_t total = uint64_t(nxh) * b.ny * b.nz;
+    for (uint64_t e = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; e < total;
+         e += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t kx = uint32_t(e % nxh);
+        const uint64_t r = e / nxh;
+        const uint32_t ky = uint32_t(r % b.ny), kz = uint32_t(r / b.ny);
+        const unsigned long long ay = min(ky, b.ny - ky), az = min(kz, b.nz - kz);
+        const long long s = shell_of((unsigned long long)kx * kx + ay * ay + az * az);
+        if (s == 0 || s >= nshell) continue;
+        const double re = double(spec[2 * e]), im = double(spec[2 * e + 1]);
+        const unsigned int wgt = (kx == 0 || (b.nx % 2 == 0 && kx == b.nx / 2)) ? 1u : 2u;
+        atomicAdd(&sums[s], wgt * (re * re + im * im) * inv_n);
+        atomicAdd(&cnts[s], (unsigned long long)wgt);
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < nshell; s += blockDim.x) {
+        if (cnts[s]) {
+            atomicAdd(&S[s], sums[s]);
+            atomicAdd(&cnt[s], cnts[s]);
+        }
+    }
+}
+
+// Whether the shells are summed element by element.
+inline bool shells_flat(const BoxDesc &b, int nshell)
+{
+    const uint64_t nxh = b.nx / 2 + 1, chunks = std::min<uint64_t>((nxh + 31) / 32, uint64_t(nshell) / 32 + 1);
+    return nxh <= 2 || (chunks >= 4 && nxh * b.ny * b.nz < 29000 * chunks);
 }
 
 // Training pairs: for every node the features x_i = g_i / sqrt(rho0 kT w_i /
@@ -804,14 +900,22 @@ cudaError_t launch_observable(const void *g, int prec, const BoxDesc &b, int obs
 cudaError_t launch_shells(const void *spec, int prec, const BoxDesc &b, int nshell, const unsigned int *peak, double *S,
                           unsigned long long *cnt, cudaStream_t s)
 {
+    const double inv_n = 1.0 / double(b.n);   // a division costs the kernels a microsecond
     auto run = [&](auto zero) {
         using T = decltype(zero);
+        if (shells_flat(b, nshell)) {
+            const uint64_t total = uint64_t(b.nx / 2 + 1) * b.ny * b.nz;
+            const int grid = int(std::min<uint64_t>((total + 255) / 256, 2048));
+            k_shells_flat<T><<<grid, 256, size_t(nshell) * (sizeof(double) + sizeof(unsigned long long)), s>>>(
+                static_cast<const T *>(spec), b, nshell, inv_n, S, cnt);
+            return;
+        }
         const int warps = shell_warps<T>(nshell);
         const uint64_t rows = uint64_t(b.ny / 2 + 1) * (b.nz / 2 + 1);
         const int grid = int(std::min<uint64_t>((rows + warps - 1) / warps, uint64_t(b.nsm) * 4));
         cudaFuncSetAttribute(k_shells<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kShellSmem));
         k_shells<T><<<grid, 32 * warps, warps * nshell * kShellBin<T>, s>>>(static_cast<const T *>(spec), b, nshell,
-                                                                            peak, S, cnt);
+                                                                            inv_n, peak, S, cnt);
     };
     if (prec == 0) run(0.0);
     else run(0.0f);

@@ -12,14 +12,22 @@ namespace flbm {
 __device__ __forceinline__ float eft_add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float eft_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float eft_mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float eft_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float eft_fms(float a, float b, float c) { return __fmaf_rn(a, b, -c); }
 __device__ __forceinline__ double eft_add(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double eft_sub(double a, double b) { return __dsub_rn(a, b); }
+// packed pairs, each lane rounded once; a - b as fma(b, -1, a)
+__device__ __forceinline__ float2 eft_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 eft_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 eft_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 eft_fms(float2 a, float2 b, float2 c)
+{
+    return __ffma2_rn(a, b, make_float2(-c.x, -c.y));
+}
 #else
 inline float eft_add(float a, float b) { return a + b; }
 inline float eft_sub(float a, float b) { return a - b; }
 inline float eft_mul(float a, float b) { return a * b; }
-inline float eft_fma(float a, float b, float c) { return fmaf(a, b, c); }
+inline float eft_fms(float a, float b, float c) { return fmaf(a, b, -c); }
 inline double eft_add(double a, double b) { return a + b; }
 inline double eft_sub(double a, double b) { return a - b; }
 #endif
@@ -40,27 +48,31 @@ __host__ __device__ __forceinline__ R two_sum(R a, R b, R &e)
 // of K terms S is within 4 K^3 2^-72 S of the exact one before it is rounded
 // to FP64 -- inside FP64's own K 2^-53 S up to 360 terms.  FP64 arithmetic
 // runs at two operations per clock and SM and bounded the spectra before.
-template <typename T> struct ShellSum;
-template <> struct ShellSum<float> {
-    float hi, mid, lo;
-    __host__ __device__ __forceinline__ void zero() { hi = mid = lo = 0.0f; }
-    __host__ __device__ __forceinline__ void add(float h, float m)
+template <typename V>
+struct TripleSum {   // V = float, or float2: two sums, a lane each
+    V hi, mid, lo;
+    __host__ __device__ __forceinline__ void add(V h, V m)
     {
-        float e, r, q;
+        V e, r, q;
         hi = two_sum(hi, h, e);
         mid = two_sum(mid, e, r);
         mid = two_sum(mid, m, q);
-        lo += r + q;
+        lo = eft_add(lo, eft_add(r, q));
     }
+    __host__ __device__ __forceinline__ void add_square(V v)
+    {
+        const V p = eft_mul(v, v);
+        add(p, eft_fms(v, v, p));
+    }
+};
+template <typename T> struct ShellSum;
+template <> struct ShellSum<float> : TripleSum<float> {
+    using TripleSum<float>::add;
+    __host__ __device__ __forceinline__ void zero() { hi = mid = lo = 0.0f; }
     __host__ __device__ __forceinline__ void add(const ShellSum &o)
     {
         add(o.hi, o.mid);
         lo += o.lo;
-    }
-    __host__ __device__ __forceinline__ void add_square(float v)
-    {
-        const float p = eft_mul(v, v);
-        add(p, eft_fma(v, v, -p));
     }
     __host__ __device__ __forceinline__ void scale2()
     {
