@@ -27,6 +27,8 @@ namespace {
 // Scratch capacity: partial sums of at most kNoallocMaxCtas CTAs (13 doubles
 // each, 208 KiB) plus 16 bytes of flags, per device.
 constexpr int kNoallocMaxCtas = 2048;
+static_assert((kDirectPairs - 1 + 31) / 32 <= kNoallocMaxCtas,
+              "boxes below kDirectPairs nodes run a CTA per 32 nodes, as many as the device holds");
 
 struct NoallocScratch {
     double partials[kNoallocMaxCtas * NSTAT];
