@@ -44,18 +44,18 @@ WORKLOAD = dict(nx=512, ny=512, nz=512, tau=0.6, kT=1e-5, rho0=1.0, seed=2026010
 BYTES_PER_NODE = {"fp32": 27 * 4 * 2, "fp16": 27 * 2 * 2, "fp64": 27 * 8 * 2}
 CS2 = 1.0 / 3.0
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_step_rows_f32_gmf_traffic.txt")
-KERNEL_SOURCES = ["step_kernel.cuh", "lattice.cuh", "internal.h", "step_f32.cu", "step_f32_paced.cu"]
+KERNEL_SOURCES = ["step_kernel.cuh", "error_free.cuh", "lattice.cuh", "internal.h", "step_f32.cu", "step_f32_paced.cu"]
 TRAFFIC16_FILE = os.path.join(ROOT, "profiles", "k_step_rows_f16_gmf_traffic.txt")
-KERNEL16_SOURCES = ["step_kernel.cuh", "lattice.cuh", "internal.h", "step_f16.cu", "step_f16_nx512.cu"]
+KERNEL16_SOURCES = ["step_kernel.cuh", "error_free.cuh", "lattice.cuh", "internal.h", "step_f16.cu", "step_f16_nx512.cu"]
 ENS_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_step_ens_f32_gmf_traffic.txt")
-ENS_KERNEL_SOURCES = ["ens_kernel.cuh", "step_kernel.cuh", "lattice.cuh", "internal.h", "stats.cuh",
+ENS_KERNEL_SOURCES = ["ens_kernel.cuh", "step_kernel.cuh", "error_free.cuh", "lattice.cuh", "internal.h", "stats.cuh",
                       "ens_f32.cu", "ens_f32p.cu"]
 LEARNED_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_step_learned_f32_traffic.txt")
 MS_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_ms_step_f32_gmf_traffic.txt")
-MS_KERNEL_SOURCES = ["mstate.cu", "step_kernel.cuh", "lattice.cuh", "internal.h"]
+MS_KERNEL_SOURCES = ["mstate.cu", "step_kernel.cuh", "error_free.cuh", "lattice.cuh", "internal.h"]
 MS_BYTES_PER_NODE = 10 * 4 * 2   # moment state: ten FP32 numbers read and written per node
-LEARNED_KERNEL_SOURCES = ["step_learned.cu", "mlp_tc.cuh", "umma.cuh", "step_kernel.cuh", "lattice.cuh",
-                          "internal.h"]
+LEARNED_KERNEL_SOURCES = ["step_learned.cu", "mlp_tc.cuh", "umma.cuh", "step_kernel.cuh", "error_free.cuh",
+                          "lattice.cuh", "internal.h"]
 
 
 def parse_args(argv=None):
