@@ -1,5 +1,5 @@
 // step_f64.cu -- FP64 instantiations of the fused step kernels (parity path:
-// double deviations, double arithmetic, double-precision log/sqrt/sincospi).
+// double deviations, double arithmetic, normals from tables).
 #include "step_kernel.cuh"
 
 namespace flbm {

@@ -780,9 +780,10 @@ __device__ __forceinline__ I pop_index(const Nbr<I> &nb, I n, I N, int i, int j,
 // memory (no barrier: no other thread touches it; and reading early is safe
 // in place, a node's AA reads are exactly its own writes), so the loads of 54
 // populations wait behind the collision instead of in front of it.
-// What bounds it: instruction issue (800-915 a node, a quarter more than the
-// row kernels, for the 108 accesses of two nodes) with 12 warps per SM; DRAM
-// at 57-64 % of its peak.  250 x 243 x 121 FP32: 326 us a step (22.5 GLUPS),
+// What bounds it: latency at the 11 warps per SM that 168 registers leave; no
+// pipe is full (issue slots 49 % busy, FMA 42 %, DRAM 56 %), with 893
+// instructions a node, a quarter more than the row kernels, for the 108
+// accesses of two nodes.  250 x 243 x 121 FP32: 326 us a step (22.5 GLUPS),
 // 374 with one node per thread in row chunks; 100^3 51 us instead of 76; 16^3
 // 8 instead of 21.  Unstaged: 332 us, and 56 us at 100^3.
 template <typename S, typename R, typename I, int SCHEME, bool ODD, bool STATS, int NP>
